@@ -192,6 +192,33 @@ int pd_fused_launch(int n, const FusedSeg *segs, int nsegs, int64_t nitems, cons
 int pd_fused_occupancy(int n, int threads, size_t qwords, int nbuf, int *blocks_per_sm);
 int pd_fused_team(int n);
 
+// The interpolation tables of one (prime, variable) with m nodes in cosets of
+// L (cinterp_kernel), Jf = m / L whole cosets and s = m % L nodes of one more:
+// word offsets of the parts, each a multiple of 4 so that rows of vt load as
+// 16-byte vectors.  All entries are Montgomery forms.
+//   vt  [Jf + 1][jp]  row j < Jf: column j of the inverse Vandermonde matrix
+//                     of z_0..z_{Jf-1} (padded with zeros to jp words); row
+//                     Jf: the coefficients of z^0..z^(Jf-1) of Pi
+//   tw1 [Jf][L]       L^-1 w^(-j r)
+//   rk  [L]           psi^-k, psi = w^(N / L)
+//   ell [Jf]          weights of the value at z_Jf: prod_{l != j} (z_Jf - z_l) / (z_j - z_l)
+//   bm  [s][s]        inverse of X[t][r] Pi(z_Jf), X[t][r] = psi^(t r) w^(Jf r), r, t < s
+//   nx  [s][L]        -bm X
+struct CiTab {
+  int jp, vt, tw1, rk, ell, bm, nx, words;
+  PD_HD CiTab(int m, int L) {
+    const int Jf = m / L, s = m % L;
+    jp = (Jf + 3) / 4 * 4;
+    vt = 0;
+    tw1 = vt + (Jf + 1) * jp;
+    rk = tw1 + (Jf * L + 3) / 4 * 4;
+    ell = rk + (L + 3) / 4 * 4;
+    bm = ell + jp;
+    nx = bm + (s * s + 3) / 4 * 4;
+    words = nx + (s * L + 3) / 4 * 4;
+  }
+};
+
 // Node exponent of node k of a variable with N points and order radix L
 // (L = 1: natural order): cosets of the L-th roots, one after another.
 PD_HD int node_exp(int k, int N, int L) { return k / L + (N / L) * (k % L); }

@@ -223,12 +223,6 @@ static int pow2_at_least(int64_t x) {
   return (int)n;
 }
 
-// Words of the interpolation tables of one variable (see polydet_plan).
-static int itab_words(int M, int L) {
-  const int Jf = M / L, s = M % L;
-  return Jf * Jf + Jf * L + L + s * L * Jf + s * s + Jf + 1;
-}
-
 // Inverse of an n x n matrix mod p by Gauss-Jordan (n < 8 here; always
 // invertible: a scaled Vandermonde matrix of distinct nodes).
 static std::vector<uint64_t> mat_inv_mod(std::vector<uint64_t> A, int n, uint64_t p) {
@@ -258,14 +252,15 @@ static std::vector<uint64_t> mat_inv_mod(std::vector<uint64_t> A, int n, uint64_
   return I;
 }
 
-// The interpolation tables of one (prime, variable), in the layout of
-// polydet_plan's comment.  They depend on (p, w, N, L, M) only and are
+// The interpolation tables of one (prime, variable), in the layout of CiTab
+// (common.cuh).  They depend on (p, w, N, L, M) only and are
 // memoised for the process.
 static void interp_tables(uint32_t p32, uint32_t w32, int N, int L, int M, uint32_t *dst) {
   static std::mutex mu;
   static std::map<std::tuple<uint32_t, uint32_t, int, int>, std::vector<uint32_t>> cache;
   const auto key = std::make_tuple(p32, w32, L, M);
-  const int words = itab_words(M, L);
+  const CiTab T(M, L);
+  const int words = T.words;
   {
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(key);
@@ -282,8 +277,8 @@ static void interp_tables(uint32_t p32, uint32_t w32, int N, int L, int M, uint3
   const uint64_t psi = pw(w, (uint64_t)(N / L)), ipsi = inv(psi);
   std::vector<uint64_t> z(Jf + 1);
   for (int j = 0; j <= Jf; ++j) z[j] = pw(w, (uint64_t)L * j);
-  uint32_t *o = dst;
-  // VfInv by Lagrange: Vf^-1[u][j] = [z^u] q_j(z) / q_j(z_j), q_j = Pi / (z - z_j)
+  memset(dst, 0, (size_t)words * sizeof(uint32_t));
+  // inverse Vandermonde by Lagrange: V^-1[u][j] = [z^u] q_j(z) / q_j(z_j), q_j = Pi / (z - z_j)
   std::vector<uint64_t> pic(Jf + 1, 0);  // Pi(z), built factor by factor
   pic[0] = 1;
   for (int j = 0; j < Jf; ++j) {
@@ -294,35 +289,37 @@ static void interp_tables(uint32_t p32, uint32_t w32, int N, int L, int M, uint3
   for (int j = 0; j < Jf; ++j) {
     qc[Jf - 1] = 1;  // q_j = Pi / (z - z_j): q_{k-1} = pi_k + z_j q_k
     for (int k = Jf - 1; k >= 1; --k) qc[k - 1] = (pic[k] + z[j] * qc[k]) % p;
-    uint64_t den = 0;
-    for (int k = Jf - 1; k >= 0; --k) den = (den * z[j] + qc[k]) % p;
+    uint64_t den = 0, top = 0;  // q_j(z_j), q_j(z_Jf)
+    for (int k = Jf - 1; k >= 0; --k) {
+      den = (den * z[j] + qc[k]) % p;
+      top = (top * z[Jf] + qc[k]) % p;
+    }
     const uint64_t id = inv(den);
-    for (int u = 0; u < Jf; ++u) o[(size_t)u * Jf + j] = mont(qc[u] * id % p);
+    for (int u = 0; u < Jf; ++u) dst[T.vt + (size_t)j * T.jp + u] = mont(qc[u] * id % p);
+    dst[T.ell + j] = mont(top * id % p);
   }
-  o += (size_t)Jf * Jf;
+  for (int u = 0; u < Jf; ++u) dst[T.vt + (size_t)Jf * T.jp + u] = mont(pic[u]);
   const uint64_t Linv = inv((uint64_t)L);
   for (int j = 0; j < Jf; ++j)
-    for (int r = 0; r < L; ++r) o[(size_t)j * L + r] = mont(Linv * inv(pw(w, (uint64_t)j * r)) % p);
-  o += (size_t)Jf * L;
-  for (int k = 0; k < L; ++k) o[k] = mont(pw(ipsi, (uint64_t)k));
-  o += L;
-  for (int t = 0; t < s; ++t)
-    for (int r = 0; r < L; ++r)
-      for (int u = 0; u < Jf; ++u)
-        o[((size_t)t * L + r) * Jf + u] =
-            mont(pw(psi, (uint64_t)t * r) * pw(w, (uint64_t)Jf * r) % p * pw(z[Jf], (uint64_t)u) % p);
-  o += (size_t)s * L * Jf;
+    for (int r = 0; r < L; ++r) dst[T.tw1 + j * L + r] = mont(Linv * inv(pw(w, (uint64_t)j * r)) % p);
+  for (int k = 0; k < L; ++k) dst[T.rk + k] = mont(pw(ipsi, (uint64_t)k));
   if (s > 0) {
     uint64_t piz = 0;  // Pi(z_Jf)
     for (int k = Jf; k >= 0; --k) piz = (piz * z[Jf] + pic[k]) % p;
-    std::vector<uint64_t> A((size_t)s * s);
+    std::vector<uint64_t> X((size_t)s * L), A((size_t)s * s);
     for (int t = 0; t < s; ++t)
-      for (int r = 0; r < s; ++r) A[(size_t)t * s + r] = pw(psi, (uint64_t)t * r) * pw(w, (uint64_t)Jf * r) % p * piz % p;
+      for (int r = 0; r < L; ++r) X[(size_t)t * L + r] = pw(psi, (uint64_t)t * r) * pw(w, (uint64_t)Jf * r) % p;
+    for (int t = 0; t < s; ++t)
+      for (int r = 0; r < s; ++r) A[(size_t)t * s + r] = X[(size_t)t * L + r] * piz % p;
     const std::vector<uint64_t> B = mat_inv_mod(A, s, p);
-    for (int i = 0; i < s * s; ++i) o[i] = mont(B[i]);
+    for (int i = 0; i < s * s; ++i) dst[T.bm + i] = mont(B[i]);
+    for (int i = 0; i < s; ++i)
+      for (int r = 0; r < L; ++r) {
+        uint64_t x = 0;
+        for (int t = 0; t < s; ++t) x = (x + B[(size_t)i * s + t] * X[(size_t)t * L + r]) % p;
+        dst[T.nx + i * L + r] = mont(p - x);
+      }
   }
-  o += (size_t)s * s;
-  for (int k = 0; k <= Jf; ++k) o[k] = mont(pic[k]);
   std::lock_guard<std::mutex> lock(mu);
   cache.emplace(key, std::vector<uint32_t>(dst, dst + words));
 }
@@ -672,21 +669,15 @@ int pd_plan_impl(polydet_plan_t *out, int n, int nvars, const int32_t *entry_deg
   // whole cosets, s = M mod L nodes of one more), P(x) = sum_r x^r Q_r(x^L)
   // and x^L = z_j = w^(L j) on coset j, so an inverse DFT of size L per coset
   // gives Q_r(z_j) and each Q_r is interpolated through z_0..z_{Jf-1}; the
-  // last s nodes fix the top coefficient of Q_r for r < s.  Per (prime,
-  // variable), Montgomery forms:
-  //   VfInv [Jf][Jf]   inverse Vandermonde of z_0..z_{Jf-1} (V[j][u] = z_j^u)
-  //   tw1   [Jf][L]    L^-1 w^(-j r)
-  //   ipsi  [L]        psi^-k, psi = w^(N / L)
-  //   H     [s][L][Jf] psi^(t r) w^(Jf r) z_Jf^u
-  //   B     [s][s]     inverse of A[t][r] = psi^(t r) w^(Jf r) Pi(z_Jf), r, t < s
-  //   pi    [Jf + 1]   coefficients of Pi(z) = prod_{j<Jf} (z - z_j)
+  // last s nodes fix the top coefficient of Q_r for r < s (Q_r = interpolant
+  // + lambda_r Pi, Pi = prod_j (z - z_j)).  Layout: CiTab (common.cuh).
   std::vector<uint32_t> itab;
   pl->full = (flags & POLYDET_FLAG_FULL_GRID) ? 1 : 0;
   if (!pl->full) {
     int off2 = 0;
     for (int v = 0; v < nvars; ++v) {
       pl->itab_off[v] = off2;
-      off2 += itab_words(pl->M[v], pl->LPo[v]);
+      off2 += CiTab(pl->M[v], pl->LPo[v]).words;
     }
     pl->itab_len = off2;
     itab.assign((size_t)nprimes * off2, 0u);
