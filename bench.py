@@ -681,7 +681,7 @@ def structured_leg(st, hbm_peak, derived_upd):
 def run_ours(args, world, rank, local):
     import torch
     from paper_2010_12117_gb300 import synth
-    from paper_2010_12117_gb300.binding import condense_steps, probe_int_peaks
+    from paper_2010_12117_gb300.binding import condense_columns, probe_int_peaks
     from paper_2010_12117_gb300.runner import BatchedRunner, PlainRunner, StageTimer
 
     torch.cuda.set_device(local)
@@ -785,23 +785,25 @@ def run_ours(args, world, rank, local):
     sms = dev_props.multi_processor_count
     sm_mhz = clocks.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     lanes = sms * 64 * sm_mhz * 1e6  # IMAD lanes per second (64 per SM per clock)
-    # The condensation kernel of order n takes its elimination steps two or
-    # three at a time (condense_steps).  One element update of a step pair
+    # The condensation kernel of order n takes its elimination steps two,
+    # three or four at a time (condense_columns).  One element update of a step pair
     # (two algorithmic updates) issues three 32x32->64-bit multiply-adds and
     # the REDC's IMAD and IMAD.HI; the pipe costs ncu measures on the probes
     # (a wide multiply-add or an IMAD.HI holds the FMA-heavy pipe two slots,
     # an IMAD one) make that 9 slots, 4.5 per update; one of a step triple
     # (three updates) four multiply-adds and the same two: 11 slots, 11/3 per
-    # update.  The probes run both element updates in registers.
-    slots = {2: 4.5, 3: 11.0 / 3.0}
-    probe_upd = {2: 2.0 * pair_s, 3: 3.0 * triple_s}
-    step_of = {n_: condense_steps(n_) for n_ in range(1, 33)}
+    # update; one of two nested pairs (four updates) five: 13 slots, 13/4 per
+    # update.  The probes run the first two element updates in registers; the
+    # third's rate is the triple's scaled by the slots.
+    slots = {2: 4.5, 3: 11.0 / 3.0, 4: 13.0 / 4.0}
+    probe_upd = {2: 2.0 * pair_s, 3: 3.0 * triple_s, 4: 4.0 * triple_s * 11.0 / 13.0}
+    step_of = {n_: condense_columns(n_) for n_ in range(1, 33)}
 
     def model_peak(n_):
         return lanes / slots[step_of[n_]]
     single_step_upd = lanes / 6.0  # the single-step kernel's model (6 slots), kept for comparison
     peak_src = (f"derived: {sms} SMs x 64 IMAD/clk x {sm_mhz:.0f} MHz / IMAD slots per update "
-                "of each order's pass (4.5 for a step pair, 11/3 for a step triple), weighted by "
+                "of each order's pass (4.5 for a step pair, 11/3 for a step triple, 13/4 for two nested pairs), weighted by "
                 "each order's updates")
     # per order: the update rate against its integer-pipe peak, the byte rate
     # against HBM, and the time either bound alone allows; the sum of those

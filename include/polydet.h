@@ -416,14 +416,18 @@ int polydet_batch_set_chunk_words(polydet_batch_t batch, uint64_t words);
  * determinant values of those items are not written.  on = 0 restores normal
  * operation.  Not during a graph capture (uploads the segment tables). */
 int polydet_batch_test_drop_copies(polydet_batch_t batch, int on);
-/* Lanes that share one determinant in the condensation kernels of order n
+/* Lanes that share one determinant in the fused kernels of order n
  * (a CTA size must be a multiple of it); POLYDET_EINVAL outside 1..32.  Host
  * only: no device call. */
 int polydet_team_size(int n);
-/* Elimination steps the condensation kernels of order n take per pass (2 or
- * 3; the instruction mix, and so the integer-pipe ceiling, depends on it);
- * POLYDET_EINVAL outside 1..32.  Host only. */
+/* Columns of the pivot blocks the condensation kernels of order n eliminate
+ * by (2 or 3); POLYDET_EINVAL outside 1..32.  Host only. */
 int polydet_condense_steps(int n);
+/* Columns the condensation kernels of order n eliminate at a time: 2 or 3, or
+ * 4 where two 2 x 2 pivot blocks are applied together (the instruction mix,
+ * and so the integer-pipe ceiling, depends on it); POLYDET_EINVAL outside
+ * 1..32.  Host only. */
+int polydet_condense_columns(int n);
 
 /* Stage 1 of a batch (Sec. 3.1): every variable but the last (fused orders)
  * or but the first (materialized orders); all orders (n = 0 in

@@ -124,6 +124,7 @@ SIGNATURES = {
                                      ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
                                      ctypes.POINTER(ctypes.c_double)]),
     "polydet_condense_steps": (_I, [_I]),
+    "polydet_condense_columns": (_I, [_I]),
     "polydet_last_error": (ctypes.c_char_p, []),
 }
 
@@ -408,7 +409,7 @@ def tail_entry_words(M) -> int:
 
 
 def team_size(n: int) -> int:
-    """Lanes per determinant in the condensation kernels of order n (a pure
+    """Lanes per determinant in the fused kernels of order n (a pure
     host query of the library's table)."""
     t = lib().polydet_team_size(int(n))
     if t < 1:
@@ -575,10 +576,18 @@ def probe_int_peaks(stream=None) -> tuple[float, float, float, float]:
 
 
 def condense_steps(n: int) -> int:
-    """Elimination steps per pass of the condensation kernels of order n."""
+    """Columns of the pivot blocks of the condensation kernels of order n (2 or 3)."""
     t = lib().polydet_condense_steps(int(n))
     if t < 1:
         _check(t, "polydet_condense_steps")
+    return t
+
+
+def condense_columns(n: int) -> int:
+    """Columns the condensation kernels of order n eliminate at a time (2, 3 or 4)."""
+    t = lib().polydet_condense_columns(int(n))
+    if t < 1:
+        _check(t, "polydet_condense_columns")
     return t
 
 

@@ -99,5 +99,9 @@ extern "C" int polydet_team_size(int n) {
 }
 
 extern "C" int polydet_condense_steps(int n) {
-  return (n >= 1 && n <= POLYDET_MAX_N) ? kStep[n] : POLYDET_EINVAL;
+  return (n >= 1 && n <= POLYDET_MAX_N) ? (kCond[n].step == 3 ? 3 : 2) : POLYDET_EINVAL;
+}
+
+extern "C" int polydet_condense_columns(int n) {
+  return (n >= 1 && n <= POLYDET_MAX_N) ? kCond[n].step : POLYDET_EINVAL;
 }

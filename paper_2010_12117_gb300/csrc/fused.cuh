@@ -35,6 +35,11 @@
 #include "bulk.cuh"
 #include "condense.cuh"
 
+template <int NN>
+struct TeamFor {
+  static constexpr int value = kTeam[NN];  // lanes per matrix
+};
+
 // Words of shared memory for the entry slices of a CTA of `threads` lanes.
 template <int NN>
 __host__ __device__ constexpr size_t fused_slice_words(int threads) {
@@ -125,17 +130,12 @@ __device__ __noinline__ uint2 fused_det(const uint32_t *mine, int bd, int t, Mod
 #pragma unroll
     for (int i = 0; i < NN; ++i) a[m][i] = (j >= 0) ? mine[(m * NN + i) * bd] : 0u;
   }
-  uint32_t Q = md.r1, den = md.r1;
-  bool zero = false;
-  if constexpr (kStep[NN] == 3) {
-    Fast3Step<NN, T, 0>::run(a, p, pinv, Q, den, zero);
-  } else {
-    Fast2Step<NN, T, 0>::run(a, p, pinv, Q, den, zero);
-    zero |= p > PD_FOLD3_MAX;  // as in condense_kernel: larger primes redo every matrix
-  }
-  if (__any_sync(PD_FULL, zero))  // a zero pivot in this warp: redo with the search
+  PivAcc sink{md.r1, md.r1, false};
+  fast_pass<NN, T, kFusedStep[NN], 0>(a, p, pinv, sink);
+  if (step_folds3(kFusedStep[NN])) sink.zero |= p > PD_FOLD3_MAX;  // as in condense_kernel
+  if (__any_sync(PD_FULL, sink.zero))  // a zero pivot in this warp: redo with the search
     return fused_det_search<NN, T>(mine, bd, t, md);
-  return make_uint2(Q, den);
+  return make_uint2(sink.Q, sink.den);
 }
 
 // Geometry of one item: its first node g0, the first of the partial-tensor

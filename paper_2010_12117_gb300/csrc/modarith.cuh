@@ -71,6 +71,17 @@ PD_D uint32_t redc4(uint64_t x, uint32_t p, uint32_t pinv) {
   return min(r, r - p);
 }
 
+// x / R mod p for x < 5 p^2 (a sum of up to five products of residues) and
+// p <= PD_FOLD3_MAX: 5 p^2 < 2^64, and the REDC value lies in (-p, 2.18 p).
+PD_D uint32_t redc5(uint64_t x, uint32_t p, uint32_t pinv) {
+  const uint32_t m = (uint32_t)x * pinv;
+  const uint32_t hi = (uint32_t)(x >> 32), mh = __umulhi(m, p);
+  uint32_t r = hi - mh;
+  r = (hi < mh) ? r + p : r;
+  r = min(r, r - p);
+  return min(r, r - p);
+}
+
 PD_D uint32_t mfms3(uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t e, uint32_t f,
                     uint32_t p, uint32_t pinv) {
   return redc3((uint64_t)a * b + (uint64_t)c * d + (uint64_t)e * f, p, pinv);

@@ -1,36 +1,52 @@
-// Per-order launch table of the condensation kernels.
+// Per-order launch tables of the condensation and fused kernels.
 #pragma once
 
 #include "../../include/polydet.h"
 
-// Lanes per matrix (T), the resident CTAs per SM the condensation kernel of
-// each order n is compiled for (its __launch_bounds__ minimum), the steps its
-// fast pass takes at a time (2: Schur complement of a 2 x 2 block,
-// Fast2Step; 3: of a 3 x 3 block, Fast3Step) and its threads per CTA.
-// First chosen per order from sweeps on GB300 with random 31-bit matrices on
-// 2^19 nodes: one lane while the whole matrix fits in registers (n <= 12),
-// then 2, 4 and 8 lanes; three steps where they beat two by 3 % or more
-// (8-25 % at the orders that take them).  Then, for orders 14-24, every
-// alternative was timed on the launches the batched workload itself makes
-// (the sweep's single large launch did not always predict them: taking rows
-// two at a time or four steps per pass won there and lost here), and the
-// table keeps what won on the workload: at n = 24 two steps on two CTAs of
-// 192 threads (4 % over three CTAs of 128; three steps on the same CTAs won
-// 2.6 % on launches of the workload's jobs in their input variable order but
-// not on the benchmark's own, so two stay), at n = 22 and 20 two steps on
-// 256-thread CTAs, at 21 three steps on 256-thread CTAs.
-// Threads per CTA: the fully unrolled elimination of the large orders is
-// longer than the instruction cache, so fewer, larger CTAs per SM, whose
-// warps walk the same code together, stall less on instruction fetch (ncu at
-// n = 24: 0.24 instead of 1.30 no-instruction stalls per issue with two CTAs
-// of 192 threads instead of three of 128, the same 12 warps and registers).
-// Orders 25-31 were not swept: they take the choice of n = 32.
+// The condensation kernel of order n (condense_kernel): lanes per matrix (T),
+// columns its fast pass takes at a time (step_at: 2 pairs, 3 triples, 4 two
+// nested pairs), the CTAs per SM it is compiled for (its __launch_bounds__
+// minimum, which sets the registers per thread), threads per CTA, and where
+// the pivots are folded into (numerator, denominator): by every lane as they
+// come (lane_pivots) or by one thread per matrix at the end.
+//
+// What bounds the kernel is the integer multiply pipe and how many warps fill
+// it: 12 to 20 warps per SM, each with its whole matrix in registers.  Chosen
+// per order by timing every candidate on three primes of 140001 random
+// matrices (and on 5329 nodes, a single wave), in microseconds, the previous
+// table's choice (pairs or triples, pivots folded by every lane) first:
+//   n = 8 41.4 -> 35.0   9 45.3 -> 43.2  10 57.4 -> 53.3  11 65.6  12 90.2 -> 82.0
+//   13 123 -> 102   14 139 -> 123   15 164 -> 145   16 204 -> 170   17 230 -> 220
+//   18 287 -> 244   19 327 -> 297   20 390 -> 338   21 450 -> 414   22 507 -> 474
+//   23 573 -> 531   24 643 -> 570   25 991 -> 667   26 1062 -> 804  27 1171 -> 858
+//   28 1223 -> 962  29 1407 -> 1312 30 1513 -> 1399 31 1684 -> 1436 32 1777 -> 1592
+// Quads (five products and one reduction for four columns) win from order 14
+// on, where the trailing matrix is large enough to pay for their panel.  Four
+// lanes beat eight up to order 28: the panel is computed once per lane, and
+// the registers that spill (up to 700 bytes at order 28) cost less; from 29
+// on they cost more (order 29: 1454 with four lanes).  Folding the pivots at
+// the end saves 5 to 9 % where a lane has registers to spare (triples, orders
+// 15 and 22 to 25) and costs as much in spills where it has not (order 16:
+// 204 instead of 171).
+struct CondCfg {
+  int team, step, ctas, threads;
+  bool lane_pivots;
+};
+constexpr CondCfg kCond[POLYDET_MAX_N + 1] = {
+    {1, 2, 1, 128, false},                                                                       // (none)
+    {1, 2, 1, 128, false}, {1, 2, 1, 128, false}, {1, 2, 1, 128, false}, {1, 2, 3, 128, false},  // 1 - 4
+    {1, 2, 2, 128, false}, {1, 2, 4, 128, false}, {1, 2, 4, 128, false}, {1, 3, 5, 128, false},  // 5 - 8
+    {1, 3, 5, 128, false}, {1, 4, 5, 128, false}, {1, 3, 4, 128, false}, {1, 3, 4, 128, false},  // 9 - 12
+    {1, 3, 3, 128, true},  {2, 4, 4, 128, true},  {2, 4, 4, 128, false}, {2, 4, 2, 256, true},   // 13 - 16
+    {2, 4, 3, 128, false}, {2, 4, 3, 128, true},  {4, 4, 4, 128, false}, {4, 4, 4, 128, true},   // 17 - 20
+    {4, 4, 4, 128, true},  {4, 4, 2, 256, false}, {4, 4, 4, 128, false}, {4, 4, 2, 192, false},  // 21 - 24
+    {4, 4, 2, 192, false}, {4, 4, 3, 128, true},  {4, 4, 3, 128, true},  {4, 4, 2, 192, false},  // 25 - 28
+    {8, 4, 3, 128, true},  {8, 4, 2, 192, true},  {8, 4, 3, 128, false}, {8, 4, 2, 192, true}};  // 29 - 32
+
+// The fused kernels (fused.cuh): lanes per matrix and columns per step.  One
+// lane while the whole matrix fits in registers (n <= 12), then 2, 4 and 8:
+// fewer lanes would need entry slices that do not fit in shared memory.
 constexpr int kTeam[POLYDET_MAX_N + 1] = {1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 1, 2, 2, 2, 2,
                                           2, 2, 2, 4, 4, 4, 4, 4, 8, 8, 8, 8, 8, 8, 8, 8};
-constexpr int kMinBlocks[POLYDET_MAX_N + 1] = {1, 1, 1, 1, 3, 2, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4, 4,
-                                               4, 3, 3, 2, 2, 2, 4, 2, 3, 3, 3, 3, 3, 3, 3, 3};
-constexpr int kStep[POLYDET_MAX_N + 1] = {2, 2, 2, 2, 2, 2, 2, 2, 3, 2, 3, 3, 3, 3, 2, 3, 2,
-                                          3, 3, 3, 2, 3, 2, 3, 2, 2, 2, 2, 2, 2, 2, 2, 2};
-constexpr int kThreads[POLYDET_MAX_N + 1] = {128, 128, 128, 128, 128, 128, 128, 128, 128, 128, 128,
-                                             128, 128, 128, 128, 128, 128, 128, 128, 128, 256, 256,
-                                             256, 128, 192, 128, 128, 128, 128, 128, 128, 128, 128};
+constexpr int kFusedStep[POLYDET_MAX_N + 1] = {2, 2, 2, 2, 2, 2, 2, 2, 3, 2, 3, 3, 3, 3, 2, 3, 2,
+                                               3, 3, 3, 2, 3, 2, 3, 2, 2, 2, 2, 2, 2, 2, 2, 2};
