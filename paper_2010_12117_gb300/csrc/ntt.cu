@@ -14,8 +14,9 @@
 // in time; the output is in natural order) and writes Lout x Ct back.  Data
 // are plain residues; twiddles are stored in Montgomery form so one REDC per
 // butterfly gives a plain product.
-#include <limits.h>
 #include <stdio.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "ntt_direct.cuh"
@@ -287,7 +288,7 @@ extern "C" int polydet_eval(polydet_plan_t pl, const int32_t *coeffs, int lo, in
 // (one 16-byte load, the same for the whole warp) and the values each serve
 // several products: 3 loads per 8 products.  One dot product per thread (two
 // loads per product) was bound by the load pipe at a quarter of the integer
-// pipe's rate: 73^3 nodes and 18 primes took 369 us, now 255 us.
+// pipe's rate: 73^3 nodes and 18 primes took 369 us, now 172 us.
 struct CiArgs {
   const uint32_t *in;
   uint32_t *out;
@@ -347,7 +348,7 @@ PD_D void small_dft(uint32_t (&x)[L], const uint32_t *rk, uint32_t p, uint32_t p
 constexpr int kCiU = 4;  // coefficients per thread and column (one 16-byte table load)
 
 template <int L>
-__global__ void __launch_bounds__(512) cinterp_kernel(CiArgs a) {
+__global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
   extern __shared__ uint32_t sm[];
   const int q = a.prime_lo + blockIdx.z;
   const ModP md = a.mod[q];
@@ -373,120 +374,123 @@ __global__ void __launch_bounds__(512) cinterp_kernel(CiArgs a) {
     const int64_t aa = (ncols >> 32) ? col / a.B : (int64_t)((uint32_t)col / (uint32_t)a.B);
     return aa * m * a.B + (col - aa * a.B);
   };
+  // a thread keeps its column through the phases (blockDim is a multiple of Ct)
+  const int c = tid & (Ct - 1), jstep = bd >> logCt;
 
   if (a.rows) {
     const uint32_t *src = in + col0 * m;
-    for (int c = tid >> 5; c < ncol; c += bd >> 5)
-      for (int r = tid & 31; r < m; r += 32) Y[c * mp + r] = src[(int64_t)c * m + r];
+    for (int k = tid >> 5; k < ncol; k += bd >> 5)
+      for (int r = tid & 31; r < m; r += 32) Y[k * mp + r] = src[(int64_t)k * m + r];
     __syncthreads();
   }
+  // the column's node values: node r at src[r * sstep]
+  const uint32_t *src = a.rows ? Y + c * mp : in + word0(c < ncol ? c : 0);
+  const int64_t sstep = a.rows ? 1 : a.B;
   // 1. inverse DFT of each whole coset, twisted
-  for (int f = tid; f < Jf << logCt; f += bd) {
-    const int j = f >> logCt, c = f & (Ct - 1);
-    uint32_t x[L];
-    if (c >= ncol) {
+  {
+    const uint32_t *sj = src + (int64_t)(tid >> logCt) * L * sstep;
+    const uint32_t *tw = tab + T.tw1 + (tid >> logCt) * L;
+    uint32_t *qj = Qv + ((tid >> logCt) << logCt) + c;
+    for (int j = tid >> logCt; j < Jf; j += jstep) {
+      uint32_t x[L];
 #pragma unroll
-      for (int t = 0; t < L; ++t) x[t] = 0u;
-    } else if (a.rows) {
+      for (int t = 0; t < L; ++t) x[t] = c < ncol ? sj[t * sstep] : 0u;
+      small_dft<L>(x, tab + T.rk, p, pinv);
 #pragma unroll
-      for (int t = 0; t < L; ++t) x[t] = Y[c * mp + j * L + t];
-    } else {
-      const uint32_t *src = in + word0(c) + (int64_t)j * L * a.B;
-#pragma unroll
-      for (int t = 0; t < L; ++t) x[t] = __ldg(src + t * a.B);
+      for (int r = 0; r < L; ++r) qj[(r * JJ) << logCt] = mmul(x[r], __ldg(tw + r), p, pinv);
+      sj += (int64_t)jstep * L * sstep;
+      tw += jstep * L;
+      qj += jstep << logCt;
     }
-    small_dft<L>(x, tab + T.rk, p, pinv);
-#pragma unroll
-    for (int r = 0; r < L; ++r)
-      Qv[((r * JJ + j) << logCt) + c] = mmul(x[r], __ldg(tab + T.tw1 + j * L + r), p, pinv);
   }
   __syncthreads();
   if (s > 0) {  // 2. the last coset
-    for (int f = tid; f < L << logCt; f += bd) {
-      const int r = f >> logCt, c = f & (Ct - 1);
-      Es[f] = dot_strided(tab + T.ell, Qv + ((r * JJ) << logCt) + c, Ct, Jf, p, pinv);
-    }
+    for (int r = tid >> logCt; r < L; r += jstep)
+      Es[(r << logCt) + c] = dot_strided(tab + T.ell, Qv + ((r * JJ) << logCt) + c, Ct, Jf, p, pinv);
     __syncthreads();
-    for (int f = tid; f < L << logCt; f += bd) {
-      const int r = f >> logCt, c = f & (Ct - 1);
+    for (int r = tid >> logCt; r < L; r += jstep) {
       uint32_t lam = 0u;
       if (r < s && c < ncol) {
         lam = dot_strided(tab + T.nx + r * L, Es + c, Ct, L, p, pinv);
-        const uint32_t *src = a.rows ? Y + c * mp + Jf * L : in + word0(c) + (int64_t)Jf * L * a.B;
-        const int64_t step = a.rows ? 1 : a.B;
-        for (int t = 0; t < s; ++t) lam = addm(lam, mmul(__ldg(tab + T.bm + r * s + t), src[t * step], p, pinv), p);
+        for (int t = 0; t < s; ++t)
+          lam = addm(lam, mmul(__ldg(tab + T.bm + r * s + t), src[(Jf * L + t) * sstep], p, pinv), p);
       }
       Qv[((r * JJ + Jf) << logCt) + c] = lam;
     }
     __syncthreads();
   }
   // 3. coefficient e = L u + r of columns c2 and c2 + Ct / 2, u = u0 .. u0 + 3
-  const int half = Ct >> 1;
+  const int half = Ct >> 1, c2 = tid & (half - 1);
   const int chunks = (Jf + kCiU - 1) / kCiU;
-  for (int f = tid; f < (chunks * L) << (logCt - 1); f += bd) {
-    const int c2 = f & (half - 1), ru = f >> (logCt - 1);
+  uint32_t *dst[2];
+  const int64_t dstep = a.rows ? 1 : a.B;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int ch = c2 + h * half;
+    dst[h] = a.rows ? Y + ch * mp : out + word0(ch < ncol ? ch : 0);
+  }
+  for (int ru = tid >> (logCt - 1); ru < chunks * L; ru += bd >> (logCt - 1)) {
     const int r = ru % L, u0 = ru / L * kCiU;
-    const uint32_t *V = tab + T.vt + u0;  // 16-byte aligned: every table offset is a multiple of 4 words
+    // 16-byte aligned: every table offset is a multiple of 4 words
+    const uint4 *V = reinterpret_cast<const uint4 *>(tab + T.vt + u0);
     const uint32_t *y = Qv + ((r * JJ) << logCt) + c2;
+    const int vstep = T.jp >> 2;
     uint32_t acc[kCiU][2];
 #pragma unroll
     for (int i = 0; i < kCiU; ++i) acc[i][0] = acc[i][1] = 0u;
-    for (int j0 = 0; j0 < JJ; j0 += 4) {  // up to four products per REDC
+    auto group = [&](auto count) {  // up to four products per REDC
+      constexpr int N = decltype(count)::value;
       uint64_t t[kCiU][2];
 #pragma unroll
-      for (int i = 0; i < kCiU; ++i) t[i][0] = t[i][1] = 0u;
+      for (int k = 0; k < N; ++k) {
+        const uint4 v4 = __ldg(V + k * vstep);
+        const uint32_t v[kCiU] = {v4.x, v4.y, v4.z, v4.w};
+        const uint32_t y0 = y[k << logCt], y1 = y[(k << logCt) + half];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (j0 + k < JJ) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4 *>(V + (int64_t)(j0 + k) * T.jp));
-          const uint32_t y0 = y[(j0 + k) << logCt], y1 = y[((j0 + k) << logCt) + half];
-          t[0][0] += (uint64_t)v.x * y0;
-          t[0][1] += (uint64_t)v.x * y1;
-          t[1][0] += (uint64_t)v.y * y0;
-          t[1][1] += (uint64_t)v.y * y1;
-          t[2][0] += (uint64_t)v.z * y0;
-          t[2][1] += (uint64_t)v.z * y1;
-          t[3][0] += (uint64_t)v.w * y0;
-          t[3][1] += (uint64_t)v.w * y1;
+        for (int i = 0; i < kCiU; ++i) {
+          t[i][0] = (uint64_t)v[i] * y0 + (k ? t[i][0] : 0ull);
+          t[i][1] = (uint64_t)v[i] * y1 + (k ? t[i][1] : 0ull);
         }
       }
+      V += N * vstep;
+      y += N << logCt;
 #pragma unroll
       for (int i = 0; i < kCiU; ++i) {
         acc[i][0] = addm(acc[i][0], redc4(t[i][0], p, pinv), p);
         acc[i][1] = addm(acc[i][1], redc4(t[i][1], p, pinv), p);
       }
-    }
+    };
+    int j = JJ;
+    for (; j >= 4; j -= 4) group(std::integral_constant<int, 4>());
+    if (j == 3) group(std::integral_constant<int, 3>());
+    if (j == 2) group(std::integral_constant<int, 2>());
+    if (j == 1) group(std::integral_constant<int, 1>());
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int c = c2 + h * half;
-      if (c >= ncol) continue;
-      if (a.rows) {
+      if (c2 + h * half >= ncol) continue;
+      uint32_t *d = dst[h] + (L * u0 + r) * dstep;
 #pragma unroll
-        for (int i = 0; i < kCiU; ++i)
-          if (u0 + i < Jf) Y[c * mp + L * (u0 + i) + r] = acc[i][h];
-      } else {
-        uint32_t *dst = out + word0(c) + (int64_t)(L * u0 + r) * a.B;
-#pragma unroll
-        for (int i = 0; i < kCiU; ++i)
-          if (u0 + i < Jf) dst[(int64_t)(L * i) * a.B] = acc[i][h];
+      for (int i = 0; i < kCiU; ++i) {
+        if (u0 + i < Jf) *d = acc[i][h];
+        d += L * dstep;
       }
     }
   }
   // the top coefficients lambda_r: e = L Jf + r, r < s
   for (int f = tid; f < s << logCt; f += bd) {
-    const int r = f >> logCt, c = f & (Ct - 1);
-    if (c >= ncol) continue;
-    const uint32_t lam = Qv[((r * JJ + Jf) << logCt) + c];
+    const int r = f >> logCt, k = f & (Ct - 1);
+    if (k >= ncol) continue;
+    const uint32_t lam = Qv[((r * JJ + Jf) << logCt) + k];
     if (a.rows)
-      Y[c * mp + L * Jf + r] = lam;
+      Y[k * mp + L * Jf + r] = lam;
     else
-      out[word0(c) + (int64_t)(L * Jf + r) * a.B] = lam;
+      out[word0(k) + (L * Jf + r) * a.B] = lam;
   }
   if (a.rows) {
     __syncthreads();
-    uint32_t *dst = out + col0 * m;
-    for (int c = tid >> 5; c < ncol; c += bd >> 5)
-      for (int r = tid & 31; r < m; r += 32) dst[(int64_t)c * m + r] = Y[c * mp + r];
+    uint32_t *o = out + col0 * m;
+    for (int k = tid >> 5; k < ncol; k += bd >> 5)
+      for (int r = tid & 31; r < m; r += 32) o[(int64_t)k * m + r] = Y[k * mp + r];
   }
 }
 
@@ -528,7 +532,7 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
     a.s = a.m % L;
     a.rows = a.B == 1;
     const int64_t ncols = a.A * a.B;
-    int ct = 64;
+    int ct = 32;
     while (ct > 2 && cinterp_words(a.m, L, ct, a.rows) * sizeof(uint32_t) > 56 * 1024) ct >>= 1;
     while (ct > 2 && ct / 2 >= ncols) ct >>= 1;
     // small passes (a job's few columns): fewer columns per CTA, so that the
@@ -539,17 +543,14 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
     if (smem > kMaxSmem) return POLYDET_EINVAL;
     a.Ct = ct;
     a.logCt = ilog2(ct);
-    // threads: the multiple of 32 whose rounds over step 3's items waste the fewest
-    const int items = (a.Jf + kCiU - 1) / kCiU * L * (ct / 2);
-    int th = 64, waste = INT_MAX;
-    for (int x = 512; x >= 128; x -= 32) {
-      const int w = (items + x - 1) / x * x - items;
-      if (items <= x ? w < waste : w + x / 8 < waste) {
-        waste = items <= x ? w : w + x / 8;
-        th = x;
-      }
-    }
-    if (items <= 64) th = 64;
+    // threads: a multiple of the columns, no more than step 3 has items for.
+    // Small CTAs, so that those of an SM are in different phases (73^3 nodes,
+    // 18 primes: 172 us with 128 threads, 180 with 192, 207 with 512; 64
+    // columns and 320 threads 186), larger ones where the grid is short of
+    // four CTAs per SM (193^2 nodes, 24 primes: 34.8 us with 256, 36.9 with 128)
+    const int64_t ctas = (ncols + ct - 1) / ct * np;
+    const int items = std::max(1, (a.Jf + kCiU - 1) / kCiU) * L * (ct / 2);
+    const int th = std::min((items + 63) / 64 * 64, ctas >= 4 * sms ? 128 : 256);
     a.in = cur;
     a.in_prime_stride = cur_prime;
     if (v == 0) {
