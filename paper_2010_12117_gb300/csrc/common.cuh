@@ -56,6 +56,7 @@ struct polydet_plan_s {
   // device tables
   ModP *d_mod;            // [P]
   uint32_t *d_tw_fwd;     // [P][tw_len]  w^j * R, per variable at offset tw_off[v]
+  uint2 *d_tw_shoup;      // [P][tw_len]  (w^j, floor(w^j 2^32 / p))
   uint32_t *d_tw_inv;     // [P][tw_len]  w^-j * R
   uint32_t *d_ninv;       // [P][nvars]   N_v^-1 * R
   uint32_t *d_rn;         // [P]          R^n mod p (condensation output scale)

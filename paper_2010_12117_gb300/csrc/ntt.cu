@@ -119,24 +119,40 @@ static int ilog2(int64_t x) {
   return l;
 }
 
+template <int CPT, class Off>
+static int launch_direct_as(const TxArgs &a, dim3 grid, cudaStream_t st) {
+  constexpr int TH = kDirectThreads;
+  switch (a.Lin) {
+    case 1: coltx_direct_kernel<1, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 2: coltx_direct_kernel<2, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 3: coltx_direct_kernel<3, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 4: coltx_direct_kernel<4, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 5: coltx_direct_kernel<5, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 6: coltx_direct_kernel<6, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 7: coltx_direct_kernel<7, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    default: coltx_direct_kernel<8, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+  }
+  PD_CUDA(cudaGetLastError());
+  return POLYDET_OK;
+}
+
 template <int CPT>
 static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes, cudaStream_t st) {
   constexpr int TH = kDirectThreads;
   dim3 grid((unsigned)((ncols + TH * CPT - 1) / (TH * CPT)), (unsigned)items, (unsigned)nprimes);
   if (a.flat_items)
     grid = dim3((unsigned)((ncols * items * a.flat_groups + TH - 1) / TH), 1u, (unsigned)nprimes);
-  switch (a.Lin) {
-    case 1: coltx_direct_kernel<1, CPT><<<grid, TH, 0, st>>>(a); break;
-    case 2: coltx_direct_kernel<2, CPT><<<grid, TH, 0, st>>>(a); break;
-    case 3: coltx_direct_kernel<3, CPT><<<grid, TH, 0, st>>>(a); break;
-    case 4: coltx_direct_kernel<4, CPT><<<grid, TH, 0, st>>>(a); break;
-    case 5: coltx_direct_kernel<5, CPT><<<grid, TH, 0, st>>>(a); break;
-    case 6: coltx_direct_kernel<6, CPT><<<grid, TH, 0, st>>>(a); break;
-    case 7: coltx_direct_kernel<7, CPT><<<grid, TH, 0, st>>>(a); break;
-    default: coltx_direct_kernel<8, CPT><<<grid, TH, 0, st>>>(a); break;
-  }
-  PD_CUDA(cudaGetLastError());
-  return POLYDET_OK;
+  // 32-bit byte offsets where all the output a CTA's base pointer covers lies
+  // within 4 GB of it (rows the kernel steps over past the last one included)
+  const int64_t rows = (int64_t)a.N + 8;
+  int64_t span;
+  if (a.il_L)
+    span = (rows * (a.B / a.il_L) + 1) * a.il_n2 * a.il_Lp;
+  else
+    span = (a.flat_items ? (int64_t)items * a.out_item_stride : 0) +
+           a.A * rows * (a.out_row ? a.out_row : a.B) + TH * CPT;
+  return span < ((int64_t)1 << 30) ? launch_direct_as<CPT, uint32_t>(a, grid, st)
+                                   : launch_direct_as<CPT, int64_t>(a, grid, st);
 }
 
 static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
@@ -149,12 +165,18 @@ static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
   const bool window_ok = a.row_hi == 0 || (a.olp > 1 && a.olp == lp_in && a.row_lo % lp_in == 0);
   if (!a.inverse && a.Lin <= 8 && a.N <= kDirectTwSmem && rows_ok && window_ok &&
       (a.olp <= 1 || a.olp == lp_in)) {
-    // columns per thread: more share each coset's twiddles, fewer leave
-    // fewer idle lanes in the last CTA of a row of B columns (measured: two
-    // per thread from rows of about 1000 columns on; four only for inputs of
-    // at most five words, whose registers still allow two CTAs per SM)
-    int cpt = a.B < 8 ? 1 : (ncols >= 8192 ? 4 : (ncols >= 1024 ? 2 : 1));
-    if (cpt == 4 && a.Lin > 5) cpt = 2;
+    // columns per thread: a warp's are consecutive, so that with more of them
+    // fewer of the sectors that rows off the 32-byte grid split are shared
+    // between warps, and they share each coset's twiddles; fewer leave fewer
+    // idle lanes at the end of a row of B columns and need fewer registers.
+    // x_1 passes in TB/s with 1 / 2 / 4: inputs of 4 words, rows of 1369
+    // columns 5.1 / 5.5 / 5.5, 3 words, 943 columns 5.4 / 5.1 / 5.7, 2 words,
+    // 441 columns 4.6 / 5.3 / 5.1, 7 words, 193 columns 3.6 / 5.4 / 2.5.  One
+    // where the columns are not one block (A > 1, interleaved output) or the
+    // pass is too small to fill the chip with more.
+    int cpt = 1;
+    if (a.A == 1 && !a.il_L && a.B >= 128 && a.B * items * nprimes >= 152 * 4096)
+      cpt = lp_in <= 4 && a.B >= ((a.out_row ? a.out_row : a.B) % 8 ? 512 : 8192) ? 4 : 2;
     // short rows (one column per thread): one grid axis over (item, column)
     // pairs, so that rows shorter than a CTA, or a row's last CTA, leave no
     // threads idle
@@ -243,6 +265,7 @@ extern "C" int polydet_eval(polydet_plan_t pl, const int32_t *coeffs, int lo, in
     a.prime_lo = lo;
     a.mod = pl->d_mod;
     a.tw = pl->d_tw_fwd;
+    a.tws = pl->d_tw_shoup;
     a.tw_len = pl->tw_len;
     a.tw_off = pl->tw_off[v];
     a.ninv = pl->d_ninv;
@@ -669,6 +692,7 @@ static TxArgs forward_pass(const polydet_plan_s *pl, int v, int lo) {
   a.prime_lo = lo;
   a.mod = pl->d_mod;
   a.tw = pl->d_tw_fwd;
+  a.tws = pl->d_tw_shoup;
   a.tw_len = pl->tw_len;
   a.tw_off = pl->tw_off[v];
   a.ninv = pl->d_ninv;
@@ -800,6 +824,7 @@ int pd_eval_partial(const polydet_plan_s *pl, const int32_t *coeffs, int lo, int
     a.prime_lo = lo;
     a.mod = pl->d_mod;
     a.tw = pl->d_tw_fwd;
+    a.tws = pl->d_tw_shoup;
     a.tw_len = pl->tw_len;
     a.tw_off = pl->tw_off[v];
     a.ninv = pl->d_ninv;

@@ -18,6 +18,7 @@ struct TxArgs {
   int prime_lo;
   const ModP *mod;
   const uint32_t *tw;
+  const uint2 *tws;  // forward passes: (w^j, floor(w^j 2^32 / p)), same offsets as tw
   int tw_len, tw_off;
   const uint32_t *ninv;
   int nvars, var;
@@ -55,24 +56,44 @@ PD_HD int out_rows(const TxArgs &a) { return a.row_hi ? a.row_hi - a.row_lo : a.
 // y = DFT_LP(c_e w^(j e))[t] with the LP-th root psi = w^(N/LP): Lin - 1
 // twiddle products and a register DFT of size LP per LP outputs, in which
 // the LP - Lin inputs that are zero are folded away at compile time.  A
-// thread owns CPT columns (kDirectThreads apart, so every store of a row
-// stays coalesced) and loads each coset's twiddles once for all of them.
+// thread owns CPT columns, 32 apart, so that a warp's columns are consecutive
+// and every store of a row is coalesced, and loads each coset's twiddles once
+// for all of them.
 // With one column per thread the grid may instead run over (item, column,
 // coset group) triples (TxArgs::flat_items): short rows then fill whole CTAs,
 // and a pass with few columns in all spreads each column's cosets over
 // several threads.
 //
-// The integer multiply pipe, which also executes much of the address and
-// move arithmetic, bounds the pass together with the write bandwidth, so the
-// loop is kept lean: the twiddle circle is staged in shared memory once per
-// CTA and read with 32-bit indices, and the cosets whose rows are all stored
-// go through one pointer per output row with the columns at fixed offsets
-// from it, without per-store predicates; only the ragged last coset takes
-// the predicated path.  Plans keep D_v <= n d_v, so with at most 8 inputs
-// (d_v <= 7) and n <= 32 a circle has N <= 256 points; launch_pass sends
-// anything longer to the shared-memory pass kernel.
+// The pass writes far more than it reads, and its bound is the write
+// bandwidth (6.0 TB/s on rows that start on 32-byte sectors) as long as the
+// instructions per word stay few and few sectors are written in parts:
+//  - a warp's columns are consecutive and its CPT stores of a row follow one
+//    another, because rows of an odd number of words split a sector at both
+//    ends of every 128-byte store: with a thread's columns a CTA apart the
+//    other part came from another warp, and a trivariate x_1 pass of 583 MB
+//    (rows of 1369 words) took 127 us, now 106 us; the same with the part
+//    arriving even later (146 us) is what a leaner loop alone gave;
+//  - a twiddle product is Shoup's: with w' = floor(w 2^32 / p) at hand,
+//    x w - umulhi(x, w') p lies in [0, 2p) for any x < 2^32, two low products
+//    and a high one where a Montgomery product needs a wide, a low and a high
+//    one; the operand may be an unreduced difference (23 -> 18 instructions
+//    per word; aligned rows 5.3 -> 6.0 TB/s);
+//  - the twiddle circle (pairs w, w') is staged in shared memory;
+//  - stores go to a base pointer that is the same for the whole CTA plus a
+//    running offset per output row, 32-bit wherever the output of a CTA's
+//    prime (flat grid) or item fits in 4 GB (Off = uint32_t, launch_pass);
+//  - the cosets whose rows are all stored take no per-store predicate.
+// Plans keep D_v <= n d_v, so with at most 8 inputs (d_v <= 7) and n <= 32 a
+// circle has N <= 256 points; launch_pass sends anything longer to the
+// shared-memory pass kernel.
 constexpr int kDirectThreads = 256;
 constexpr int kDirectTwSmem = 256;
+
+// x w mod p in [0, p), tw = (w, floor(w 2^32 / p)), any x < 2^32.
+PD_D uint32_t smul(uint32_t x, uint2 tw, uint32_t p) {
+  const uint32_t r = x * tw.x - __umulhi(x, tw.y) * p;
+  return min(r, r - p);
+}
 
 // x + y and x - y mod p where ZX / ZY say that x / y is known to be zero.
 template <bool ZX, bool ZY>
@@ -102,143 +123,82 @@ PD_D void dft4(const uint32_t (&x)[4], uint32_t (&y)[4], uint32_t r4, uint32_t p
   y[3] = sub_z<ZA, ZB>(a1, b1, p);
 }
 
+// The same with a Shoup pair for the root; the product takes the difference
+// x1 - x3 + p unreduced.
+template <bool Z0, bool Z1, bool Z2, bool Z3>
+PD_D void dft4s(const uint32_t (&x)[4], uint32_t (&y)[4], uint2 r4, uint32_t p) {
+  const uint32_t a0 = add_z<Z0, Z2>(x[0], x[2], p), a1 = sub_z<Z0, Z2>(x[0], x[2], p);
+  constexpr bool ZA = Z0 && Z2, ZB = Z1 && Z3;
+  const uint32_t b0 = add_z<Z1, Z3>(x[1], x[3], p);
+  const uint32_t b1 = ZB ? 0u : smul(Z3 ? x[1] : x[1] + p - x[3], r4, p);
+  y[0] = add_z<ZA, ZB>(a0, b0, p);
+  y[2] = sub_z<ZA, ZB>(a0, b0, p);
+  y[1] = add_z<ZA, ZB>(a1, b1, p);
+  y[3] = sub_z<ZA, ZB>(a1, b1, p);
+}
+
 template <int LIN>
 struct DirectLP {
   static constexpr int value = LIN <= 1 ? 1 : LIN <= 2 ? 2 : LIN <= 4 ? 4 : 8;
 };
 
-// The outputs y[k][t] of coset j for the thread's CPT columns (TW(k): the
-// twiddle w^k in Montgomery form).
-template <int LIN, int CPT, class Tw>
-PD_D void direct_coset(int j, const uint32_t (&c)[CPT][LIN], uint32_t (&y)[CPT][DirectLP<LIN>::value],
-                       const Tw &TW, uint32_t r1, uint32_t r4, uint32_t psi1, uint32_t psi2, uint32_t psi3,
-                       uint32_t p, uint32_t pinv) {
+// The roots of the register DFT: psi^1, psi^2, psi^3 of order 8 (psi^2 alone
+// of order 4).
+struct DirectRoots {
+  uint2 psi1, psi2, psi3;
+};
+
+// The outputs y[t] of a coset with twiddles w[e] = w^(j e) for one column.
+template <int LIN>
+PD_D void direct_coset(const uint32_t (&c)[LIN], const uint2 (&w)[LIN], uint32_t (&y)[DirectLP<LIN>::value],
+                       const DirectRoots &rt, uint32_t p) {
   constexpr int LP = DirectLP<LIN>::value;
-  uint32_t w[LIN];
-  w[0] = r1;
+  uint32_t z[LP];
+  z[0] = c[0];
 #pragma unroll
-  for (int e = 1; e < LIN; ++e) w[e] = TW(j * e);
+  for (int e = 1; e < LP; ++e) z[e] = (e < LIN) ? smul(c[e % LIN], w[e % LIN], p) : 0u;
+  if constexpr (LP == 1) {
+    y[0] = z[0];
+  } else if constexpr (LP == 2) {
+    y[0] = addm(z[0], z[1], p);
+    y[1] = subm(z[0], z[1], p);
+  } else if constexpr (LP == 4) {
+    dft4s<false, false, (LIN <= 2), (LIN <= 3)>(z, y, rt.psi2, p);
+  } else {
+    // even and odd halves, then y_t = E_t + psi^t O_t, y_{t+4} = E_t - psi^t O_t
+    const uint32_t xe[4] = {z[0], z[2], z[4], z[6]}, xo[4] = {z[1], z[3], z[5], z[7]};
+    uint32_t E[4], O[4];
+    dft4s<false, false, (LIN <= 4), (LIN <= 6)>(xe, E, rt.psi2, p);
+    dft4s<false, (LIN <= 3), (LIN <= 5), (LIN <= 7)>(xo, O, rt.psi2, p);
+    O[1] = smul(O[1], rt.psi1, p);
+    O[2] = smul(O[2], rt.psi2, p);
+    O[3] = smul(O[3], rt.psi3, p);
 #pragma unroll
-  for (int k = 0; k < CPT; ++k) {
-    uint32_t z[LP];
-    z[0] = c[k][0];
-#pragma unroll
-    for (int e = 1; e < LP; ++e) z[e] = (e < LIN) ? mmul(w[e], c[k][e], p, pinv) : 0u;
-    if (LP == 1) {
-      y[k][0] = z[0];
-    } else if (LP == 2) {
-      y[k][0] = add_z<false, LIN < 2>(z[0], z[1 % LP], p);
-      y[k][1 % LP] = sub_z<false, LIN < 2>(z[0], z[1 % LP], p);
-    } else if (LP == 4) {
-      uint32_t x[4] = {z[0], z[1 % LP], z[2 % LP], z[3 % LP]}, yy[4];
-      dft4<false, false, (LIN <= 2), (LIN <= 3)>(x, yy, r4, p, pinv);
-#pragma unroll
-      for (int t = 0; t < 4; ++t) y[k][t % LP] = yy[t];
-    } else {
-      // even and odd halves, then y_t = E_t + psi^t O_t, y_{t+4} = E_t - psi^t O_t
-      uint32_t xe[4] = {z[0], z[2 % LP], z[4 % LP], z[6 % LP]};
-      uint32_t xo[4] = {z[1 % LP], z[3 % LP], z[5 % LP], z[7 % LP]};
-      uint32_t E[4], O[4];
-      dft4<false, false, (LIN <= 4), (LIN <= 6)>(xe, E, r4, p, pinv);
-      dft4<false, (LIN <= 3), (LIN <= 5), (LIN <= 7)>(xo, O, r4, p, pinv);
-      const uint32_t t1 = mmul(psi1, O[1], p, pinv);
-      const uint32_t t2 = mmul(psi2, O[2], p, pinv);
-      const uint32_t t3 = mmul(psi3, O[3], p, pinv);
-      y[k][0] = addm(E[0], O[0], p);
-      y[k][4 % LP] = subm(E[0], O[0], p);
-      y[k][1 % LP] = addm(E[1], t1, p);
-      y[k][5 % LP] = subm(E[1], t1, p);
-      y[k][2 % LP] = addm(E[2], t2, p);
-      y[k][6 % LP] = subm(E[2], t2, p);
-      y[k][3 % LP] = addm(E[3], t3, p);
-      y[k][7 % LP] = subm(E[3], t3, p);
+    for (int t = 0; t < 4; ++t) {
+      y[t] = addm(E[t], O[t], p);
+      y[t + 4] = subm(E[t], O[t], p);
     }
   }
 }
 
-// Cosets [jlo, jhi) of the thread's columns: the full ones (j < jfull)
-// through the row pointers rp[t] = op[0] + toff[t] (fast_store: all CPT
-// columns exist and lie kDirectThreads words apart in the output), the rest
-// predicated per store.
-template <int LIN, int CPT, class Tw>
-PD_D void direct_cosets(const TxArgs &a, const Tw &TW, const uint32_t (&c)[CPT][LIN], uint32_t *(&op)[CPT],
-                        bool fast_store, int jlo, int jhi, int64_t ostride, uint32_t r1, uint32_t p,
-                        uint32_t pinv) {
-  constexpr int LP = DirectLP<LIN>::value;
-  const int N = a.N;
-  const int J = N / LP;
-  uint32_t r4 = 0u, psi1 = 0u, psi2 = 0u, psi3 = 0u;
-  if (LP >= 4) r4 = TW(N >> 2);  // w^(N/4), a primitive 4th root
-  if (LP == 8) {
-    psi1 = TW(N >> 3);
-    psi2 = r4;
-    psi3 = TW(3 * (N >> 3));
-  }
-  // Natural order (olp <= 1): coset j holds rows j + J t, stored while
-  // j < lim[t].  Coset order (olp == LP): coset j holds rows j LP + t, so
-  // only the cosets of the stored rows are computed: those of
-  // [row_lo, row_hi) (row_lo a multiple of LP), whose first one lands in
-  // output row 0.
-  const bool coset_rows = a.olp > 1;
-  const int rhi = a.row_hi ? a.row_hi : a.Lout;
-  int lim[LP];
-  int64_t toff[LP];  // words from a coset's first row to its row t
-#pragma unroll
-  for (int t = 0; t < LP; ++t) {
-    lim[t] = coset_rows ? rhi - t : a.Lout - J * t;
-    toff[t] = (int64_t)(coset_rows ? t : J * t) * ostride;
-  }
-  const int64_t jstep = (int64_t)(coset_rows ? LP : 1) * ostride;  // next coset's first row
-  int jfull = fast_store ? (coset_rows ? rhi / LP : a.Lout - J * (LP - 1)) : jlo;
-  jfull = max(jlo, min(jhi, jfull));
-  if (jfull > jlo) {
-    uint32_t *rp[LP];
-#pragma unroll
-    for (int t = 0; t < LP; ++t) rp[t] = op[0] + toff[t];
-    for (int j = jlo; j < jfull; ++j) {
-      uint32_t y[CPT][LP];
-      direct_coset<LIN, CPT>(j, c, y, TW, r1, r4, psi1, psi2, psi3, p, pinv);
-#pragma unroll
-      for (int t = 0; t < LP; ++t) {
-#pragma unroll
-        for (int k = 0; k < CPT; ++k) rp[t][k * kDirectThreads] = y[k][t];
-        rp[t] += jstep;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < CPT; ++k) op[k] += (int64_t)(jfull - jlo) * jstep;
-  }
-  for (int j = jfull; j < jhi; ++j) {
-    uint32_t y[CPT][LP];
-    direct_coset<LIN, CPT>(j, c, y, TW, r1, r4, psi1, psi2, psi3, p, pinv);
-    const int jr = coset_rows ? j * LP : j;  // compared with lim[t]
-#pragma unroll
-    for (int k = 0; k < CPT; ++k) {
-      if (op[k]) {
-#pragma unroll
-        for (int t = 0; t < LP; ++t)
-          if (jr < lim[t]) op[k][toff[t]] = y[k][t];
-        op[k] += jstep;
-      }
-    }
-  }
-}
-
-template <int LIN, int CPT>
+// Off: the type of byte offsets into the output (see above).
+template <int LIN, int CPT, class Off>
 __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) {
   constexpr int LP = DirectLP<LIN>::value;
-  __shared__ uint32_t s_tw[kDirectTwSmem];
+  __shared__ uint2 s_tw[kDirectTwSmem];
   const int q = a.prime_lo + blockIdx.z;
-  const uint32_t *tw = a.tw + (size_t)q * a.tw_len + a.tw_off;
+  const uint2 *tw = a.tws + (size_t)q * a.tw_len + a.tw_off;
   // every twiddle index used is below N (j < N / LP and e < LP), and
   // N <= kDirectTwSmem (launch_pass); staged before any thread leaves
   for (int i = threadIdx.x; i < a.N; i += kDirectThreads) s_tw[i] = __ldg(tw + i);
   __syncthreads();
-  const ModP md = a.mod[q];
-  const uint32_t p = md.p, pinv = md.pinv;
+  const uint32_t p = a.mod[q].p;
   const int64_t ncols = a.A * a.B;
   int64_t item, col0;
   int grp = 0;
+  // the CTA's output: its prime's, or its item's
+  char *base = reinterpret_cast<char *>(a.out + (int64_t)blockIdx.z * a.out_prime_stride);
+  Off ibase = 0;
   if (a.flat_items) {  // CPT == 1; items * ncols * groups < 2^31 (launch_pass)
     const int gc = (int)(blockIdx.x * kDirectThreads + threadIdx.x);
     if (gc >= a.flat_items * (int)ncols * a.flat_groups) return;
@@ -246,25 +206,25 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
     grp = gc - pair * a.flat_groups;
     item = pair / (int)ncols;
     col0 = pair - item * ncols;
+    if (!a.il_L) ibase = (Off)(4 * item * a.out_item_stride);
   } else {
     item = blockIdx.y;
-    col0 = (int64_t)blockIdx.x * kDirectThreads * CPT + threadIdx.x;
+    col0 = (int64_t)blockIdx.x * kDirectThreads * CPT + (threadIdx.x >> 5) * (32 * CPT) + (threadIdx.x & 31);
     if (col0 >= ncols) return;
+    if (!a.il_L) base += 4 * (int64_t)blockIdx.y * a.out_item_stride;
   }
   const int64_t in_base = (int64_t)blockIdx.z * a.in_prime_stride + item * a.in_item_stride;
-  int64_t ostride;
-  if (a.il_L)
-    ostride = (a.B / a.il_L) * a.il_n2 * a.il_Lp;  // row r -> row index r * (B / L)
-  else
-    ostride = a.out_row ? a.out_row : a.B;
+  // bytes between output rows
+  const Off ostride = (Off)(4 * (a.il_L ? (a.B / a.il_L) * a.il_n2 * a.il_Lp  // row r -> row index r * (B / L)
+                                        : a.out_row ? a.out_row : a.B));
   uint32_t c[CPT][LIN];
-  uint32_t *op[CPT];  // output row 0 of each column (null past the last column)
-  bool all_cols = true;
+  Off op[CPT];  // output row 0 of each column
+  int nc = 0;   // columns that exist
 #pragma unroll
   for (int k = 0; k < CPT; ++k) {
-    const int64_t col = col0 + (int64_t)k * kDirectThreads;
+    const int64_t col = col0 + 32 * k;
     const bool ok = col < ncols;
-    all_cols = all_cols && ok;
+    nc += ok;
     const int64_t cc = ok ? col : col0;
     const int64_t aa = (a.A == 1) ? 0 : cc / a.B, bb = cc - aa * a.B;
     const bool zero_item = a.zero_item_plus1 && item >= a.zero_item_plus1 - 1;
@@ -275,33 +235,81 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
                           : (a.in_is_i32 ? reduce_i32(((const int32_t *)a.in)[idx], p)
                                          : ((const uint32_t *)a.in)[idx]);
     }
-    int64_t obase;
     if (a.il_L)
-      obase = (int64_t)blockIdx.z * a.out_prime_stride + ((bb / a.il_L) * a.il_n2 + item) * a.il_Lp +
-              bb % a.il_L;
+      op[k] = (Off)(4 * (((bb / a.il_L) * a.il_n2 + item) * a.il_Lp + bb % a.il_L));
     else
-      obase = (int64_t)blockIdx.z * a.out_prime_stride + item * a.out_item_stride +
-              aa * out_rows(a) * ostride + bb;
-    op[k] = ok ? a.out + obase : nullptr;
+      op[k] = ibase + (Off)(4 * (aa * out_rows(a) * (int64_t)(a.out_row ? a.out_row : a.B) + bb));
   }
-  // with one block of columns (A == 1) and the plain layout, column k sits
-  // k * kDirectThreads words after column 0 in every row
-  const bool fast_store = all_cols && a.A == 1 && !a.il_L;
   const bool coset_rows = a.olp > 1;
+  const int N = a.N, J = N / LP;
   const int rhi = a.row_hi ? a.row_hi : a.Lout;
   const int jbeg = coset_rows ? a.row_lo / LP : 0;
-  const int jend = coset_rows ? (rhi + LP - 1) / LP : a.N / LP;
+  const int jend = coset_rows ? (rhi + LP - 1) / LP : J;
+  // Natural order (olp <= 1): coset j holds rows j + J t, stored while
+  // j < lim[t].  Coset order (olp == LP): coset j holds rows j LP + t, so
+  // only the cosets of the stored rows are computed: those of
+  // [row_lo, row_hi) (row_lo a multiple of LP), whose first one lands in
+  // output row 0.
+  const Off tstep = (Off)(coset_rows ? 1 : J) * ostride;   // a coset's row t to row t + 1
+  const Off jstep = (Off)(coset_rows ? LP : 1) * ostride;  // next coset's first row
   int jlo = jbeg, jhi = jend;  // this thread's cosets
   if (a.flat_items && a.flat_groups > 1) {
     const int nj = jend - jbeg;
     const int per = (nj + a.flat_groups - 1) / a.flat_groups;
     jlo = jbeg + min(nj, grp * per);
     jhi = jbeg + min(nj, (jlo - jbeg) + per);
-    const int64_t jstep = (int64_t)(coset_rows ? LP : 1) * ostride;
 #pragma unroll
-    for (int k = 0; k < CPT; ++k)
-      if (op[k]) op[k] += (jlo - jbeg) * jstep;
+    for (int k = 0; k < CPT; ++k) op[k] += (Off)(jlo - jbeg) * jstep;
   }
-  auto TW = [&](int k) -> uint32_t { return s_tw[k]; };  // w^k R: the whole circle
-  direct_cosets<LIN, CPT>(a, TW, c, op, fast_store, jlo, jhi, ostride, md.r1, p, pinv);
+  DirectRoots rt = {};
+  if (LP >= 4) rt.psi2 = s_tw[N >> 2];  // w^(N/4), a primitive 4th root
+  if (LP == 8) {
+    rt.psi1 = s_tw[N >> 3];
+    rt.psi3 = s_tw[3 * (N >> 3)];
+  }
+  auto twiddles = [&](int j, uint2 (&w)[LIN]) {
+#pragma unroll
+    for (int e = 1; e < LIN; ++e) w[e] = s_tw[j * e];
+  };
+  // the full cosets: every column exists, and column k sits 32 k words after
+  // column 0 in every row (with more than one, launch_pass sees to one block
+  // of columns in the plain layout)
+  int j = jlo;
+  if (nc == CPT) {
+    const int jfull = min(jhi, coset_rows ? rhi / LP : a.Lout - J * (LP - 1));
+    Off ro[LP];
+#pragma unroll
+    for (int t = 0; t < LP; ++t) ro[t] = op[0] + (Off)t * tstep;
+    for (; j < jfull; ++j) {
+      uint2 w[LIN];
+      twiddles(j, w);
+      uint32_t y[CPT][LP];
+#pragma unroll
+      for (int k = 0; k < CPT; ++k) direct_coset<LIN>(c[k], w, y[k], rt, p);
+#pragma unroll
+      for (int t = 0; t < LP; ++t)
+#pragma unroll
+        for (int k = 0; k < CPT; ++k) reinterpret_cast<uint32_t *>(base + ro[t])[32 * k] = y[k][t];
+#pragma unroll
+      for (int t = 0; t < LP; ++t) ro[t] += jstep;
+    }
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) op[k] += (Off)(j - jlo) * jstep;
+  }
+  for (; j < jhi; ++j) {  // ragged cosets and the other layouts: a predicate per store
+    uint2 w[LIN];
+    twiddles(j, w);
+#pragma unroll
+    for (int k = 0; k < CPT; ++k) {
+      if (k >= nc) break;
+      uint32_t y[LP];
+      direct_coset<LIN>(c[k], w, y, rt, p);
+#pragma unroll
+      for (int t = 0; t < LP; ++t) {
+        const bool st = coset_rows ? j * LP + t < rhi : j + J * t < a.Lout;
+        if (st) *reinterpret_cast<uint32_t *>(base + op[k] + (Off)t * tstep) = y[t];
+      }
+      op[k] += jstep;
+    }
+  }
 }

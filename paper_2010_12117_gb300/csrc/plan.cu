@@ -564,6 +564,7 @@ int pd_plan_impl(polydet_plan_t *out, int n, int nvars, const int32_t *entry_deg
   // Primes, roots, Montgomery constants, twiddles.
   std::vector<ModP> mod(nprimes);
   std::vector<uint32_t> twf((size_t)nprimes * pl->tw_len, 0), twi((size_t)nprimes * pl->tw_len, 0);
+  std::vector<uint2> tws((size_t)nprimes * pl->tw_len, make_uint2(0u, 0u));
   std::vector<uint32_t> ninv((size_t)nprimes * nvars), rn(nprimes);
   for (int q = 0; q < nprimes; ++q) {
     uint32_t p = table[q];
@@ -584,6 +585,7 @@ int pd_plan_impl(polydet_plan_t *out, int n, int nvars, const int32_t *entry_deg
       for (int j = 0; j < N; ++j) {
         twf[(size_t)q * pl->tw_len + pl->tw_off[v] + j] = h_mont(x, p);
         twi[(size_t)q * pl->tw_len + pl->tw_off[v] + j] = h_mont(y, p);
+        tws[(size_t)q * pl->tw_len + pl->tw_off[v] + j] = make_uint2(x, (uint32_t)(((uint64_t)x << 32) / p));
         x = h_mulmod(x, w, p);
         y = h_mulmod(y, wi, p);
       }
@@ -695,7 +697,7 @@ int pd_plan_impl(polydet_plan_t *out, int n, int nvars, const int32_t *entry_deg
   Packer pk;
   const size_t o_mod = pk.add(mod), o_twf = pk.add(twf), o_twi = pk.add(twi), o_ninv = pk.add(ninv),
                o_rn = pk.add(rn), o_gar = pk.add(garner), o_mh = pk.add(H), o_mf = pk.add(M),
-               o_itab = pk.add(itab);
+               o_itab = pk.add(itab), o_tws = pk.add(tws);
   TableArena *arena = nullptr;
   int arc = table_arena(&arena);
   if (arc) {
@@ -723,6 +725,7 @@ int pd_plan_impl(polydet_plan_t *out, int n, int nvars, const int32_t *entry_deg
   pl->d_mod = reinterpret_cast<ModP *>(b + o_mod);
   pl->d_tw_fwd = reinterpret_cast<uint32_t *>(b + o_twf);
   pl->d_tw_inv = reinterpret_cast<uint32_t *>(b + o_twi);
+  pl->d_tw_shoup = reinterpret_cast<uint2 *>(b + o_tws);
   pl->d_ninv = reinterpret_cast<uint32_t *>(b + o_ninv);
   pl->d_rn = reinterpret_cast<uint32_t *>(b + o_rn);
   pl->d_garner = reinterpret_cast<uint32_t *>(b + o_gar);

@@ -101,3 +101,59 @@ def test_condense_residues_at_the_ends(n):
         pl.condense(evals_tensor(mats, pl.G), q, q + 1, det)
         want = [modular.det_mod_p(mats[0, g].astype(object).tolist(), p) for g in range(pl.G)]
         assert _u32(det).tolist() == want, (n, p)
+
+
+def _check_nodes(pl, terms, got, nodes, q):
+    """``got(g)`` against the sum of ``terms`` (coefficient, exponents) at
+    node g of prime q."""
+    p, ws = pl.primes[q], pl.roots[q]
+    for g in nodes:
+        s = [pl.node_exps[v][i] for v, i in enumerate(modular.grid_index(g, pl.M))]
+        want = sum(c * pow(ws[0], s[0] * e[0], p) * pow(ws[1], s[1] * e[1], p) *
+                   (pow(ws[2], s[2] * e[2], p) if len(e) > 2 else 1) for c, e in terms) % p
+        assert got(g) == want, (q, g)
+
+
+@pytest.mark.parametrize("lin", range(1, 9))
+@pytest.mark.parametrize("rows,full", [(361, False), (545, False), (544, False), (97, False), (4, True)])
+def test_eval_x1_pass(lin, rows, full):
+    """The first variable's pass with 1 to 8 coefficients: one, two and four
+    columns per thread, rows on and off the 32-byte grid, ragged ends of rows
+    and of cosets, and the power-of-two grid."""
+    from paper_2010_12117_gb300.binding import Plan
+    n, P = 24, 3
+    d2 = max(1, -(-(rows - 1) // n))
+    D1 = n * (lin - 1) - (3 if lin > 2 else 0)
+    pl = Plan(n, (lin - 1, d2), P, full_grid=full, det_degs=(D1, rows - 1))
+    rng = np.random.default_rng(100 * lin + rows)
+    c = rng.integers(-2 ** 31, 2 ** 31, (n * n, lin, d2 + 1)).astype(np.int32)
+    coeffs = torch.from_numpy(c.reshape(-1)).cuda()
+    evals = torch.empty(P * n * n * pl.G, dtype=torch.int32, device="cuda")
+    pl.eval(coeffs, 0, P, evals, pl.workspace(P))
+    ev = evals.reshape(P, n * n, pl.G)
+    nodes = sorted({0, pl.M[1] - 1, pl.G - pl.M[1], pl.G - 1, *(int(x) for x in rng.integers(0, pl.G, 12))})
+    for q in (0, P - 1):
+        for e in (0, int(rng.integers(1, n * n - 1)), n * n - 1):
+            row = _u32(ev[q, e])
+            terms = [(int(c[e, i, j]), (i, j)) for i in range(lin) for j in range(d2 + 1)]
+            _check_nodes(pl, terms, lambda g: int(row[g]), nodes, q)
+
+
+def test_eval_rows_beyond_32_bit_offsets():
+    """One entry of 15 x 8191 x 8191 nodes: its rows span more than 4 GB."""
+    from paper_2010_12117_gb300.binding import Plan
+    n, degs = 2, (7, 4095, 4095)
+    pl = Plan(n, degs, 1)
+    pl.set_entry_map(np.array([0, -1, -1, 0], dtype=np.int32), 1)
+    rng = np.random.default_rng(8)
+    terms = [(int(rng.integers(-2 ** 31, 2 ** 31)), tuple(int(rng.integers(0, d + 1)) for d in degs)) for _ in range(6)]
+    coeffs = torch.zeros([d + 1 for d in degs], dtype=torch.int32, device="cuda")
+    for c, e in terms:
+        coeffs[e] = c
+    evals = torch.empty(pl.entries * pl.G, dtype=torch.int32, device="cuda")
+    pl.eval(coeffs.reshape(-1), 0, 1, evals, pl.workspace(1))
+    assert int(evals[pl.G:].count_nonzero()) == 0  # the zero entry
+    nodes = [0, pl.G - 1, *(int(x) for x in rng.integers(0, pl.G, 60))]
+    got = evals[torch.tensor(nodes, device="cuda")].cpu().numpy().view(np.uint32)
+    at = dict(zip(nodes, got.tolist()))
+    _check_nodes(pl, terms, at.__getitem__, nodes, 0)
