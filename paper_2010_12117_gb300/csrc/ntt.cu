@@ -119,18 +119,18 @@ static int ilog2(int64_t x) {
   return l;
 }
 
-template <int CPT, class Off>
+template <int CPT, class Off, bool FLAT>
 static int launch_direct_as(const TxArgs &a, dim3 grid, cudaStream_t st) {
   constexpr int TH = kDirectThreads;
   switch (a.Lin) {
-    case 1: coltx_direct_kernel<1, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    case 2: coltx_direct_kernel<2, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    case 3: coltx_direct_kernel<3, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    case 4: coltx_direct_kernel<4, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    case 5: coltx_direct_kernel<5, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    case 6: coltx_direct_kernel<6, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    case 7: coltx_direct_kernel<7, CPT, Off><<<grid, TH, 0, st>>>(a); break;
-    default: coltx_direct_kernel<8, CPT, Off><<<grid, TH, 0, st>>>(a); break;
+    case 1: coltx_direct_kernel<1, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 2: coltx_direct_kernel<2, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 3: coltx_direct_kernel<3, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 4: coltx_direct_kernel<4, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 5: coltx_direct_kernel<5, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 6: coltx_direct_kernel<6, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 7: coltx_direct_kernel<7, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    default: coltx_direct_kernel<8, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
   }
   PD_CUDA(cudaGetLastError());
   return POLYDET_OK;
@@ -151,8 +151,14 @@ static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes,
   else
     span = (a.flat_items ? (int64_t)items * a.out_item_stride : 0) +
            a.A * rows * (a.out_row ? a.out_row : a.B) + TH * CPT;
-  return span < ((int64_t)1 << 30) ? launch_direct_as<CPT, uint32_t>(a, grid, st)
-                                   : launch_direct_as<CPT, int64_t>(a, grid, st);
+  const bool near = span < ((int64_t)1 << 30);
+  if constexpr (CPT == 1) {
+    if (a.flat_items)
+      return near ? launch_direct_as<CPT, uint32_t, true>(a, grid, st)
+                  : launch_direct_as<CPT, int64_t, true>(a, grid, st);
+  }
+  return near ? launch_direct_as<CPT, uint32_t, false>(a, grid, st)
+              : launch_direct_as<CPT, int64_t, false>(a, grid, st);
 }
 
 static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
@@ -169,18 +175,23 @@ static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
     // fewer of the sectors that rows off the 32-byte grid split are shared
     // between warps, and they share each coset's twiddles; fewer leave fewer
     // idle lanes at the end of a row of B columns and need fewer registers.
-    // x_1 passes in TB/s with 1 / 2 / 4: inputs of 4 words, rows of 1369
-    // columns 5.1 / 5.5 / 5.5, 3 words, 943 columns 5.4 / 5.1 / 5.7, 2 words,
-    // 441 columns 4.6 / 5.3 / 5.1, 7 words, 193 columns 3.6 / 5.4 / 2.5.  One
+    // x_1 passes in TB/s with 1 / 2 / 4 columns: 4 words, rows of 1369 columns
+    // 5.1 / 5.5 / 5.6, 3 words, 943 columns 5.4 / 5.1 / 5.7, 2 words, 441
+    // columns 4.6 / 5.9 / 5.4, 7 words, 193 columns 3.6 / 5.2 / 4.3, 5 words,
+    // 97 columns 4.2 / 4.7 / 2.3, 4 words, 73 columns 4.8 / 4.2 / 3.0; on the
+    // grid (1024 columns) 5.0 / 6.0 / 5.9.  One column, over a flattened grid,
     // where the columns are not one block (A > 1, interleaved output) or the
-    // pass is too small to fill the chip with more.
+    // pass is too small to fill the chip otherwise.
     int cpt = 1;
-    if (a.A == 1 && !a.il_L && a.B >= 128 && a.B * items * nprimes >= 152 * 4096)
-      cpt = lp_in <= 4 && a.B >= ((a.out_row ? a.out_row : a.B) % 8 ? 512 : 8192) ? 4 : 2;
-    // short rows (one column per thread): one grid axis over (item, column)
-    // pairs, so that rows shorter than a CTA, or a row's last CTA, leave no
-    // threads idle
-    a.flat_items = (cpt == 1 && ncols * items < ((int64_t)1 << 31) - 256) ? items : 0;
+    bool flat = ncols * items < ((int64_t)1 << 31) - kDirectThreads;
+    if (a.A == 1 && !a.il_L && a.B >= 64 && a.B * items * nprimes >= 152 * 4096) {
+      const bool split = (a.out_row ? a.out_row : a.B) % 8;  // rows off the 32-byte grid
+      flat = false;
+      cpt = lp_in <= 4 && a.B >= (split ? 512 : 8192) ? 4 : lp_in > 4 || a.B >= 128 ? 2 : 1;
+    }
+    // short rows: one grid axis over (item, column) pairs, so that rows
+    // shorter than a CTA, or a row's last CTA, leave no threads idle
+    a.flat_items = flat ? items : 0;
     // few columns in all (a job's first pass): cut each column's cosets into
     // groups until the grid holds about 152 x 1024 threads
     a.flat_groups = 1;

@@ -71,7 +71,7 @@ PD_HD int out_rows(const TxArgs &a) { return a.row_hi ? a.row_hi - a.row_lo : a.
 //    another, because rows of an odd number of words split a sector at both
 //    ends of every 128-byte store: with a thread's columns a CTA apart the
 //    other part came from another warp, and a trivariate x_1 pass of 583 MB
-//    (rows of 1369 words) took 127 us, now 106 us; the same with the part
+//    (rows of 1369 words) took 127 us, now 104 us; the same with the part
 //    arriving even later (146 us) is what a leaner loop alone gave;
 //  - a twiddle product is Shoup's: with w' = floor(w 2^32 / p) at hand,
 //    x w - umulhi(x, w') p lies in [0, 2p) for any x < 2^32, two low products
@@ -181,8 +181,9 @@ PD_D void direct_coset(const uint32_t (&c)[LIN], const uint2 (&w)[LIN], uint32_t
   }
 }
 
-// Off: the type of byte offsets into the output (see above).
-template <int LIN, int CPT, class Off>
+// Off: the type of byte offsets into the output (see above).  FLAT (CPT == 1):
+// the grid's x axis runs over the columns of all items (TxArgs::flat_items).
+template <int LIN, int CPT, class Off, bool FLAT>
 __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) {
   constexpr int LP = DirectLP<LIN>::value;
   __shared__ uint2 s_tw[kDirectTwSmem];
@@ -194,26 +195,25 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
   __syncthreads();
   const uint32_t p = a.mod[q].p;
   const int64_t ncols = a.A * a.B;
-  int64_t item, col0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int grp = 0;
+  int64_t item = blockIdx.y;
+  // the first column, the others 32 apart
+  int64_t first = (int64_t)blockIdx.x * kDirectThreads * CPT + warp * (32 * CPT) + lane;
   // the CTA's output: its prime's, or its item's
   char *base = reinterpret_cast<char *>(a.out + (int64_t)blockIdx.z * a.out_prime_stride);
-  Off ibase = 0;
-  if (a.flat_items) {  // CPT == 1; items * ncols * groups < 2^31 (launch_pass)
-    const int gc = (int)(blockIdx.x * kDirectThreads + threadIdx.x);
-    if (gc >= a.flat_items * (int)ncols * a.flat_groups) return;
-    const int pair = gc / a.flat_groups;
-    grp = gc - pair * a.flat_groups;
+  if (FLAT) {  // items * ncols * groups < 2^31 (launch_pass)
+    const int pair = (int)first / a.flat_groups;
+    grp = (int)first - pair * a.flat_groups;
     item = pair / (int)ncols;
-    col0 = pair - item * ncols;
-    if (!a.il_L) ibase = (Off)(4 * item * a.out_item_stride);
+    first = pair - item * ncols;
+    if (item >= a.flat_items) return;
   } else {
-    item = blockIdx.y;
-    col0 = (int64_t)blockIdx.x * kDirectThreads * CPT + (threadIdx.x >> 5) * (32 * CPT) + (threadIdx.x & 31);
-    if (col0 >= ncols) return;
-    if (!a.il_L) base += 4 * (int64_t)blockIdx.y * a.out_item_stride;
+    if (first >= ncols) return;
+    if (!a.il_L) base += 4 * item * a.out_item_stride;
   }
   const int64_t in_base = (int64_t)blockIdx.z * a.in_prime_stride + item * a.in_item_stride;
+  const bool zero_item = a.zero_item_plus1 && item >= a.zero_item_plus1 - 1;
   // bytes between output rows
   const Off ostride = (Off)(4 * (a.il_L ? (a.B / a.il_L) * a.il_n2 * a.il_Lp  // row r -> row index r * (B / L)
                                         : a.out_row ? a.out_row : a.B));
@@ -222,12 +222,10 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
   int nc = 0;   // columns that exist
 #pragma unroll
   for (int k = 0; k < CPT; ++k) {
-    const int64_t col = col0 + 32 * k;
-    const bool ok = col < ncols;
+    const bool ok = first + 32 * k < ncols;
     nc += ok;
-    const int64_t cc = ok ? col : col0;
-    const int64_t aa = (a.A == 1) ? 0 : cc / a.B, bb = cc - aa * a.B;
-    const bool zero_item = a.zero_item_plus1 && item >= a.zero_item_plus1 - 1;
+    const int64_t col = ok ? first + 32 * k : first;
+    const int64_t aa = (a.A == 1) ? 0 : col / a.B, bb = col - aa * a.B;
 #pragma unroll
     for (int e = 0; e < LIN; ++e) {
       const int64_t idx = in_base + (aa * LIN + e) * a.B + bb;
@@ -238,7 +236,8 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
     if (a.il_L)
       op[k] = (Off)(4 * (((bb / a.il_L) * a.il_n2 + item) * a.il_Lp + bb % a.il_L));
     else
-      op[k] = ibase + (Off)(4 * (aa * out_rows(a) * (int64_t)(a.out_row ? a.out_row : a.B) + bb));
+      op[k] = (Off)(4 * ((FLAT ? item * a.out_item_stride : 0) +
+                         aa * out_rows(a) * (int64_t)(a.out_row ? a.out_row : a.B) + bb));
   }
   const bool coset_rows = a.olp > 1;
   const int N = a.N, J = N / LP;
@@ -253,7 +252,7 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
   const Off tstep = (Off)(coset_rows ? 1 : J) * ostride;   // a coset's row t to row t + 1
   const Off jstep = (Off)(coset_rows ? LP : 1) * ostride;  // next coset's first row
   int jlo = jbeg, jhi = jend;  // this thread's cosets
-  if (a.flat_items && a.flat_groups > 1) {
+  if (FLAT && a.flat_groups > 1) {
     const int nj = jend - jbeg;
     const int per = (nj + a.flat_groups - 1) / a.flat_groups;
     jlo = jbeg + min(nj, grp * per);
@@ -271,11 +270,11 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
 #pragma unroll
     for (int e = 1; e < LIN; ++e) w[e] = s_tw[j * e];
   };
-  // the full cosets: every column exists, and column k sits 32 k words after
-  // column 0 in every row (with more than one, launch_pass sees to one block
-  // of columns in the plain layout)
+  // the full cosets: column k sits 32 k words after column 0 in every row (with
+  // more than one, launch_pass sees to one block of columns in the plain
+  // layout); only the stores of a row's missing last columns are predicated
   int j = jlo;
-  if (nc == CPT) {
+  {
     const int jfull = min(jhi, coset_rows ? rhi / LP : a.Lout - J * (LP - 1));
     Off ro[LP];
 #pragma unroll
@@ -289,14 +288,15 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
 #pragma unroll
       for (int t = 0; t < LP; ++t)
 #pragma unroll
-        for (int k = 0; k < CPT; ++k) reinterpret_cast<uint32_t *>(base + ro[t])[32 * k] = y[k][t];
+        for (int k = 0; k < CPT; ++k)
+          if (k == 0 || k < nc) reinterpret_cast<uint32_t *>(base + ro[t])[32 * k] = y[k][t];
 #pragma unroll
       for (int t = 0; t < LP; ++t) ro[t] += jstep;
     }
 #pragma unroll
     for (int k = 0; k < CPT; ++k) op[k] += (Off)(j - jlo) * jstep;
   }
-  for (; j < jhi; ++j) {  // ragged cosets and the other layouts: a predicate per store
+  for (; j < jhi; ++j) {  // ragged cosets: a predicate per store
     uint2 w[LIN];
     twiddles(j, w);
 #pragma unroll
