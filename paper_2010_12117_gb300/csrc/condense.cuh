@@ -533,31 +533,41 @@ static inline size_t condense_reserve_bytes(int ctas) {
   return (size_t)per_sm / (size_t)(ctas + 1) + 1024;
 }
 
+template <int NN, bool FEW>
+static int condense_launch(const polydet_plan_s *pl, const uint32_t *evals, EvLayout lay, int64_t G,
+                           int64_t det_stride, int prime_lo, int nprimes, uint32_t *detvals,
+                           int ctas_per_sm, cudaStream_t st) {
+  constexpr CondCfg cfg = FEW ? cond_few(NN) : kCond[NN];
+  constexpr int T = cfg.team, threads = cfg.threads;
+  auto kern = condense_kernel<NN, T, cfg.step, cfg.ctas, threads, cfg.lane_pivots>;
+  const size_t reserve = condense_reserve_bytes(ctas_per_sm);
+  if (reserve) {
+    static PdPerDevice attr;
+    const int rc = pd_once_per_device(attr, [&] {
+      PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+      return POLYDET_OK;
+    });
+    if (rc) return rc;
+  }
+  const int64_t teams_per_cta = threads / T;
+  EntryOff<NN> off;
+  for (int e = 0; e < NN * NN; ++e) off.o[e] = (int64_t)pl->ent[e] * lay.entry;
+  dim3 grid((unsigned)((G + teams_per_cta - 1) / teams_per_cta), (unsigned)nprimes);
+  kern<<<grid, threads, reserve, st>>>(evals, detvals, G, det_stride, lay, (int64_t)pl->nent * lay.entry,
+                                       pl->d_mod, pl->d_rn, prime_lo, off);
+  PD_CUDA(cudaGetLastError());
+  return POLYDET_OK;
+}
+
 template <int NN, int HI>
 static int condense_dispatch(const polydet_plan_s *pl, const uint32_t *evals, EvLayout lay,
                              int64_t G, int64_t det_stride, int prime_lo, int nprimes,
                              uint32_t *detvals, int ctas_per_sm, cudaStream_t st) {
   if (pl->n == NN) {
-    constexpr CondCfg cfg = kCond[NN];
-    constexpr int T = cfg.team, threads = cfg.threads;
-    auto kern = condense_kernel<NN, T, cfg.step, cfg.ctas, threads, cfg.lane_pivots>;
-    const size_t reserve = condense_reserve_bytes(ctas_per_sm);
-    if (reserve) {
-      static PdPerDevice attr;
-      const int rc = pd_once_per_device(attr, [&] {
-        PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        return POLYDET_OK;
-      });
-      if (rc) return rc;
-    }
-    const int64_t teams_per_cta = threads / T;
-    EntryOff<NN> off;
-    for (int e = 0; e < NN * NN; ++e) off.o[e] = (int64_t)pl->ent[e] * lay.entry;
-    dim3 grid((unsigned)((G + teams_per_cta - 1) / teams_per_cta), (unsigned)nprimes);
-    kern<<<grid, threads, reserve, st>>>(evals, detvals, G, det_stride, lay, (int64_t)pl->nent * lay.entry,
-                                         pl->d_mod, pl->d_rn, prime_lo, off);
-    PD_CUDA(cudaGetLastError());
-    return POLYDET_OK;
+    if constexpr (!cond_same(cond_few(NN), kCond[NN]))
+      if (G * nprimes <= kCondFew)
+        return condense_launch<NN, true>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
+    return condense_launch<NN, false>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
   }
   if constexpr (NN < HI)
     return condense_dispatch<NN + 1, HI>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals,

@@ -43,6 +43,28 @@ constexpr CondCfg kCond[POLYDET_MAX_N + 1] = {
     {4, 4, 2, 192, false}, {4, 4, 3, 128, true},  {4, 4, 3, 128, true},  {4, 4, 2, 192, false},  // 25 - 28
     {8, 4, 3, 128, true},  {8, 4, 2, 192, true},  {8, 4, 3, 128, false}, {8, 4, 2, 192, true}};  // 29 - 32
 
+// Launches of at most kCondFew matrices, about one wave, take as long as one
+// matrix does, or as the wave's last CTA: for some orders more lanes, fewer
+// columns at a time or smaller CTAs than large launches like.  In
+// microseconds, the large launches' choice / this one: 100 matrices, order 16
+// 10.4 / 8.9, 30 17.5 / 15.5, 8 to 10 4.1 / 3.9, 4.7 / 4.5, 5.4 / 5.1; 16 k
+// matrices, order 25 43.1 / 41.0, 27 48.1 / 47.5, 28 57.2 / 51.5 (four lanes
+// take nearly twice as long as eight with one matrix per warp).
+constexpr int64_t kCondFew = 128 * 152;
+constexpr CondCfg cond_few(int n) {
+  return n == 8 || n == 10   ? CondCfg{1, 3, 4, 128, true}
+         : n == 9            ? CondCfg{1, 2, 4, 128, true}
+         : n == 13           ? CondCfg{2, 3, 4, 128, true}
+         : n == 16           ? CondCfg{2, 2, 4, 128, true}
+         : n >= 25 && n <= 28 ? CondCfg{8, 4, 4, 128, true}
+         : n == 30           ? CondCfg{8, 2, 3, 128, true}
+                             : kCond[n];
+}
+constexpr bool cond_same(CondCfg a, CondCfg b) {
+  return a.team == b.team && a.step == b.step && a.ctas == b.ctas && a.threads == b.threads &&
+         a.lane_pivots == b.lane_pivots;
+}
+
 // The fused kernels (fused.cuh): lanes per matrix and columns per step.  One
 // lane while the whole matrix fits in registers (n <= 12), then 2, 4 and 8:
 // fewer lanes would need entry slices that do not fit in shared memory.
