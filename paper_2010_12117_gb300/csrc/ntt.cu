@@ -381,7 +381,10 @@ PD_D void small_dft(uint32_t (&x)[L], const uint32_t *rk, uint32_t p, uint32_t p
 
 constexpr int kCiU = 4;  // coefficients per thread and column (one 16-byte table load)
 
-template <int L>
+// U: coefficients per thread, kCiU, or 1 where a pass is too small to fill the
+// chip and its time is one thread's chain of products (24 x 24 univariate, two
+// primes: interpolation + CRT 7.1 us with four, 6.0 with one).
+template <int L, int U>
 __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
   extern __shared__ uint32_t sm[];
   const int q = a.prime_lo + blockIdx.z;
@@ -453,9 +456,9 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
     }
     __syncthreads();
   }
-  // 3. coefficient e = L u + r of columns c2 and c2 + Ct / 2, u = u0 .. u0 + 3
+  // 3. coefficient e = L u + r of columns c2 and c2 + Ct / 2, u = u0 .. u0 + U - 1
   const int half = Ct >> 1, c2 = tid & (half - 1);
-  const int chunks = (Jf + kCiU - 1) / kCiU;
+  const int chunks = (Jf + U - 1) / U;
   uint32_t *dst[2];
   const int64_t dstep = a.rows ? 1 : a.B;
 #pragma unroll
@@ -464,24 +467,28 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
     dst[h] = a.rows ? Y + ch * mp : out + word0(ch < ncol ? ch : 0);
   }
   for (int ru = tid >> (logCt - 1); ru < chunks * L; ru += bd >> (logCt - 1)) {
-    const int r = ru % L, u0 = ru / L * kCiU;
-    // 16-byte aligned: every table offset is a multiple of 4 words
-    const uint4 *V = reinterpret_cast<const uint4 *>(tab + T.vt + u0);
+    const int r = ru % L, u0 = ru / L * U;
+    const uint32_t *V = tab + T.vt + u0;  // U == 4: 16-byte aligned, every table offset is a multiple of 4 words
     const uint32_t *y = Qv + ((r * JJ) << logCt) + c2;
-    const int vstep = T.jp >> 2;
-    uint32_t acc[kCiU][2];
+    const int vstep = T.jp;
+    uint32_t acc[U][2];
 #pragma unroll
-    for (int i = 0; i < kCiU; ++i) acc[i][0] = acc[i][1] = 0u;
+    for (int i = 0; i < U; ++i) acc[i][0] = acc[i][1] = 0u;
     auto group = [&](auto count) {  // up to four products per REDC
       constexpr int N = decltype(count)::value;
-      uint64_t t[kCiU][2];
+      uint64_t t[U][2];
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const uint4 v4 = __ldg(V + k * vstep);
-        const uint32_t v[kCiU] = {v4.x, v4.y, v4.z, v4.w};
+        uint32_t v[U];
+        if constexpr (U == 4) {
+          const uint4 v4 = __ldg(reinterpret_cast<const uint4 *>(V + k * vstep));
+          v[0] = v4.x, v[1] = v4.y, v[2] = v4.z, v[3] = v4.w;
+        } else {
+          v[0] = __ldg(V + k * vstep);
+        }
         const uint32_t y0 = y[k << logCt], y1 = y[(k << logCt) + half];
 #pragma unroll
-        for (int i = 0; i < kCiU; ++i) {
+        for (int i = 0; i < U; ++i) {
           t[i][0] = (uint64_t)v[i] * y0 + (k ? t[i][0] : 0ull);
           t[i][1] = (uint64_t)v[i] * y1 + (k ? t[i][1] : 0ull);
         }
@@ -489,7 +496,7 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
       V += N * vstep;
       y += N << logCt;
 #pragma unroll
-      for (int i = 0; i < kCiU; ++i) {
+      for (int i = 0; i < U; ++i) {
         acc[i][0] = addm(acc[i][0], redc4(t[i][0], p, pinv), p);
         acc[i][1] = addm(acc[i][1], redc4(t[i][1], p, pinv), p);
       }
@@ -504,7 +511,7 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
       if (c2 + h * half >= ncol) continue;
       uint32_t *d = dst[h] + (L * u0 + r) * dstep;
 #pragma unroll
-      for (int i = 0; i < kCiU; ++i) {
+      for (int i = 0; i < U; ++i) {
         if (u0 + i < Jf) *d = acc[i][h];
         d += L * dstep;
       }
@@ -544,10 +551,14 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
   PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   static PdPerDevice attr;
   const int arc = pd_once_per_device(attr, [] {
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<1, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<2, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<4, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<8, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
     return POLYDET_OK;
   });
   if (arc) return arc;
@@ -583,7 +594,9 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
     // columns and 320 threads 186), larger ones where the grid is short of
     // four CTAs per SM (193^2 nodes, 24 primes: 34.8 us with 256, 36.9 with 128)
     const int64_t ctas = (ncols + ct - 1) / ct * np;
-    const int items = std::max(1, (a.Jf + kCiU - 1) / kCiU) * L * (ct / 2);
+    int items = std::max(1, (a.Jf + kCiU - 1) / kCiU) * L * (ct / 2);
+    const bool small = ctas * items < 256 * sms;
+    if (small) items = std::max(1, a.Jf) * L * (ct / 2);
     const int th = std::min((items + 63) / 64 * 64, ctas >= 4 * sms ? 128 : 256);
     a.in = cur;
     a.in_prime_stride = cur_prime;
@@ -599,11 +612,20 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
     a.tab = pl->d_itab + pl->itab_off[v];
     a.tab_len = pl->itab_len;
     dim3 grid((unsigned)((ncols + ct - 1) / ct), 1, (unsigned)np);
-    switch (L) {
-      case 1: cinterp_kernel<1><<<grid, th, smem, st>>>(a); break;
-      case 2: cinterp_kernel<2><<<grid, th, smem, st>>>(a); break;
-      case 4: cinterp_kernel<4><<<grid, th, smem, st>>>(a); break;
-      default: cinterp_kernel<8><<<grid, th, smem, st>>>(a); break;
+    if (small) {
+      switch (L) {
+        case 1: cinterp_kernel<1, 1><<<grid, th, smem, st>>>(a); break;
+        case 2: cinterp_kernel<2, 1><<<grid, th, smem, st>>>(a); break;
+        case 4: cinterp_kernel<4, 1><<<grid, th, smem, st>>>(a); break;
+        default: cinterp_kernel<8, 1><<<grid, th, smem, st>>>(a); break;
+      }
+    } else {
+      switch (L) {
+        case 1: cinterp_kernel<1, kCiU><<<grid, th, smem, st>>>(a); break;
+        case 2: cinterp_kernel<2, kCiU><<<grid, th, smem, st>>>(a); break;
+        case 4: cinterp_kernel<4, kCiU><<<grid, th, smem, st>>>(a); break;
+        default: cinterp_kernel<8, kCiU><<<grid, th, smem, st>>>(a); break;
+      }
     }
     PD_CUDA(cudaGetLastError());
     cur = a.out;
