@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -246,6 +247,11 @@ def _stream(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
     return ctypes.c_void_p(s.cuda_stream)
 
 
+_SHAPES_KEPT = 256
+_shape_consts: dict = {}
+_shape_lock = threading.Lock()
+
+
 class Plan:
     """A polydet plan: n x n matrices in len(degs) variables, entry degree
     <= degs[v] in x_v, over the first ``nprimes`` primes of the table; node
@@ -282,17 +288,43 @@ class Plan:
         self.interp_ws_words = int(info.interp_ws_words)
         self.entries = int(info.entries)  # entries per prime of the evals tensor
         self.items = self.entries - 1 if info.unique >= 0 else self.entries  # evaluated entries
-        pr = (ctypes.c_uint32 * self.P)()
-        _check(L.polydet_plan_primes(h, pr), "polydet_plan_primes")
-        self.primes = list(pr)
-        rt = (ctypes.c_uint32 * (self.P * self.k))()
-        _check(L.polydet_plan_roots(h, rt), "polydet_plan_roots")
-        self.roots = [list(rt[q * self.k:(q + 1) * self.k]) for q in range(self.P)]
-        self.node_exps = []  # node k of x_v is root_v ** node_exps[v][k]
-        for v in range(self.k):
-            ex = (ctypes.c_int32 * max(1, self.M[v]))()
-            _check(L.polydet_plan_nodes(h, v, ex), "polydet_plan_nodes")
-            self.node_exps.append(list(ex[:self.M[v]]))
+        # primes, roots and node exponents depend on the shape alone: asked for
+        # once per shape (three library calls and hundreds of list items), kept
+        # for the most recent ones
+        key = (self.n, self.d, self.D, self.P, self.full_grid)
+        consts = _shape_consts.get(key)
+        if consts is None:
+            pr = (ctypes.c_uint32 * self.P)()
+            _check(L.polydet_plan_primes(h, pr), "polydet_plan_primes")
+            rt = (ctypes.c_uint32 * (self.P * self.k))()
+            _check(L.polydet_plan_roots(h, rt), "polydet_plan_roots")
+            exps = []  # node k of x_v is root_v ** exps[v][k]
+            for v in range(self.k):
+                ex = (ctypes.c_int32 * max(1, self.M[v]))()
+                _check(L.polydet_plan_nodes(h, v, ex), "polydet_plan_nodes")
+                exps.append(tuple(ex[:self.M[v]]))
+            consts = (tuple(pr), [tuple(rt[q * self.k:(q + 1) * self.k]) for q in range(self.P)], exps)
+            with _shape_lock:
+                while len(_shape_consts) >= _SHAPES_KEPT:
+                    _shape_consts.pop(next(iter(_shape_consts)))
+                _shape_consts[key] = consts
+        self.primes = list(consts[0])
+        self._consts = consts
+        self._roots = self._node_exps = None
+
+    @property
+    def roots(self) -> List[List[int]]:
+        """Per prime and variable, the root w_v of the nodes."""
+        if self._roots is None:
+            self._roots = [list(r) for r in self._consts[1]]
+        return self._roots
+
+    @property
+    def node_exps(self) -> List[List[int]]:
+        """Node k of x_v is root_v ** node_exps[v][k]."""
+        if self._node_exps is None:
+            self._node_exps = [list(e) for e in self._consts[2]]
+        return self._node_exps
 
     def set_entry_map(self, entry_map: np.ndarray, U: int) -> None:
         """Evaluate only the U distinct entries (map [n*n], -1 = zero entry):

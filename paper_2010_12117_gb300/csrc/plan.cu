@@ -879,8 +879,8 @@ extern "C" int polydet_sync_status(polydet_plan_t pl, void *stream, uint32_t *st
   if (!pl) return POLYDET_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   uint32_t s = 0;
+  // one wait for the copy and the reset behind it
   PD_CUDA(cudaMemcpyAsync(&s, pl->d_status, sizeof s, cudaMemcpyDeviceToHost, st));
-  PD_CUDA(cudaStreamSynchronize(st));
   PD_CUDA(cudaMemsetAsync(pl->d_status, 0, sizeof(uint32_t), st));
   PD_CUDA(cudaStreamSynchronize(st));
   if (status_out) *status_out = s;

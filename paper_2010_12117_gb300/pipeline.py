@@ -60,6 +60,15 @@ def prime_count(coeffs: np.ndarray) -> int:
     return hadamard_primes(entry_l1(coeffs))[0]
 
 
+def grid_size(n: int, degs: Sequence[int], det_degs: Optional[Sequence[int]], full_grid: bool) -> int:
+    """Evaluation nodes per prime of a plan of this shape."""
+    G = 1
+    for v, d in enumerate(degs):
+        D = n * int(d) if det_degs is None else int(det_degs[v])
+        G *= 1 << max(D, int(d)).bit_length() if full_grid else D + 1
+    return G
+
+
 def _chunk(plan: Plan, budget_bytes: int) -> int:
     per_prime = 4 * (plan.entries * plan.G + plan.G + max(plan.eval_ws_words, plan.interp_ws_words))
     return max(1, min(plan.P, budget_bytes // max(1, per_prime)))
@@ -96,28 +105,23 @@ def determinant(coeffs: np.ndarray, degs: Sequence[int], nprimes: Optional[int] 
         raise ValueError("coefficients must fit in int32")
     degs = tuple(int(d) for d in degs)
     P = nprimes if nprimes is not None else prime_count(coeffs)
+    D = det_degree_bound(entry_degrees(coeffs, degs), len(degs)) if tight_degrees else None
+    unique = unique_entries_of(coeffs.reshape(n, n, -1)) if unique_entries else None
+    if streamed is None:  # before a plan is made: the two forms take the variables in different orders
+        entries = unique[1] + 1 if unique_entries else n * n
+        streamed = 4 * (entries + 1) * grid_size(n, degs, D, full_grid) > budget_bytes
     order = list(range(len(degs)))
-    if streamed is not False:
+    if streamed:  # the plain path keeps the caller's order
         order = sorted(order, key=lambda v: (degs[v], v))
     cp = permute_coeffs(coeffs, degs, order)
     dp = tuple(degs[v] for v in order)
-    D = None
-    if tight_degrees:
-        D = det_degree_bound(entry_degrees(cp, dp), len(dp))
+    if D is not None:
+        D = tuple(D[v] for v in order)
     plan = Plan(n, dp, P, full_grid=full_grid, det_degs=D)
     rows = np.ascontiguousarray(cp, dtype=np.int32).reshape(n * n, -1)
     if unique_entries:
-        emap, U, uniq = unique_entries_of(cp)
+        emap, U, rows = unique if order == sorted(order) else unique_entries_of(cp)
         plan.set_entry_map(emap, U)
-        rows = uniq
-    if streamed is None:
-        streamed = 4 * (plan.entries * plan.G + plan.G) > budget_bytes
-    if not streamed and order != sorted(order):  # the plain path keeps the caller's order
-        plan.close()
-        return determinant(coeffs, degs, nprimes=P, store=store, budget_bytes=budget_bytes,
-                           stream=stream, stop_after_chunks=stop_after_chunks, full_grid=full_grid,
-                           tight_degrees=tight_degrees, unique_entries=unique_entries, streamed=False,
-                           as_ints=as_ints, early_stop=early_stop)
     dev = torch.device("cuda")
     st = stream if stream is not None else torch.cuda.current_stream()
     with torch.cuda.stream(st):

@@ -11,6 +11,7 @@ CUDA events on the launching stream so per-kernel time can be attributed.
 from __future__ import annotations
 
 from collections import defaultdict
+from contextlib import nullcontext
 from typing import Dict, List, Optional, Sequence
 
 import numpy as np
@@ -58,6 +59,11 @@ class StageTimer:
 def condense_updates(n: int) -> int:
     """Fused modular updates of one n x n elimination: sum_c (n-1-c)^2."""
     return (n - 1) * n * (2 * n - 1) // 6
+
+
+def _on(stream: torch.cuda.Stream):
+    """torch.cuda.stream(stream), or nothing to enter where it is current already."""
+    return nullcontext() if torch.cuda.current_stream() == stream else torch.cuda.stream(stream)
 
 
 class PlainRunner:
@@ -117,7 +123,7 @@ class PlainRunner:
 
     # -- the three phases ----------------------------------------------------
     def upload(self, stream: torch.cuda.Stream) -> None:
-        with torch.cuda.stream(stream):
+        with _on(stream):
             self.coeffs_dev.copy_(self.host_in, non_blocking=True)
 
     def compute(self, stream: torch.cuda.Stream, timer: Optional[StageTimer] = None) -> None:
@@ -126,21 +132,19 @@ class PlainRunner:
             res = self.residues[self.res_off[i]:self.res_off[i + 1]]
             n2 = pm.n * pm.n
             for lo, hi in self.chunks[i]:
-                np_ = hi - lo
                 r = res[lo * pl.C:hi * pl.C]
-                calls = [
-                    ("eval", lambda: pl.eval(c, lo, hi, self.evals, self.ws, stream),
-                     4.0 * np_ * n2 * (pl.E + pl.G), pl.k),
-                    ("condense", lambda: pl.condense(self.evals, lo, hi, self.detvals, stream),
-                     float(np_ * pl.G * condense_updates(pm.n)), 1),
-                    ("interp", lambda: pl.interp(self.detvals, lo, hi, r, self.ws, stream),
-                     4.0 * np_ * (pl.G + pl.C), pl.k),
-                ]
-                for name, fn, work, nl in calls:
-                    if timer is None:
-                        fn()
-                    else:
-                        timer.run(name, stream, fn, work, nl, tag=pm.n)
+                if timer is None:
+                    pl.eval(c, lo, hi, self.evals, self.ws, stream)
+                    pl.condense(self.evals, lo, hi, self.detvals, stream)
+                    pl.interp(self.detvals, lo, hi, r, self.ws, stream)
+                    continue
+                np_ = hi - lo
+                timer.run("eval", stream, lambda: pl.eval(c, lo, hi, self.evals, self.ws, stream),
+                          4.0 * np_ * n2 * (pl.E + pl.G), pl.k, tag=pm.n)
+                timer.run("condense", stream, lambda: pl.condense(self.evals, lo, hi, self.detvals, stream),
+                          float(np_ * pl.G * condense_updates(pm.n)), 1, tag=pm.n)
+                timer.run("interp", stream, lambda: pl.interp(self.detvals, lo, hi, r, self.ws, stream),
+                          4.0 * np_ * (pl.G + pl.C), pl.k, tag=pm.n)
             lb = self.limbs[self.limb_off[i]:self.limb_off[i + 1]]
             fn = lambda: pl.crt(res, lb, stream)  # noqa: E731
             if timer is None:
@@ -149,7 +153,7 @@ class PlainRunner:
                 timer.run("crt", stream, fn, 4.0 * pl.C * (pl.P + pl.W), 1)
 
     def download(self, stream: torch.cuda.Stream) -> None:
-        with torch.cuda.stream(stream):
+        with _on(stream):
             self.host_out.copy_(self.limbs, non_blocking=True)
 
     def check_status(self, stream: torch.cuda.Stream) -> None:
@@ -277,7 +281,7 @@ class BatchedRunner:
         return tot + len(fused)
 
     def upload(self, stream: torch.cuda.Stream) -> None:
-        with torch.cuda.stream(stream):
+        with _on(stream):
             self.coeffs_dev.copy_(self.host_in, non_blocking=True)
 
     def _stages(self, stream):
@@ -323,7 +327,7 @@ class BatchedRunner:
 
     def download(self, stream: torch.cuda.Stream) -> None:
         self._last_host = self.host_out
-        with torch.cuda.stream(stream):
+        with _on(stream):
             self.host_out.copy_(self.limbs, non_blocking=True)
 
     def run_pipelined(self, steps: int, stream: torch.cuda.Stream,
