@@ -7,11 +7,13 @@ is newer than them.
 """
 from __future__ import annotations
 
+import hashlib
 import os
 import shutil
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
+from functools import lru_cache
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -40,6 +42,18 @@ def _headers():
     out = [os.path.join(ROOT, "include", f) for f in os.listdir(os.path.join(ROOT, "include"))]
     out += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     return out
+
+
+@lru_cache(maxsize=1)
+def source_id() -> str:
+    """Identity of the kernels: a hash of every source, header and compiler flag
+    (the library itself is large and differs between two builds of one source)."""
+    h = hashlib.sha256(repr((KERNEL_RANGES, ARCH, FLAGS[:-1])).encode())
+    for path in sorted([os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cu")] + _headers()):
+        h.update(os.path.basename(path).encode())
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
 
 
 def _stale(obj: str, src: str, headers) -> bool:

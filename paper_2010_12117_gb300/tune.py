@@ -12,8 +12,10 @@ alone in each admissible configuration:
 
 It keeps the fastest and records the choice in a JSON cache keyed by device
 name, matrix order and a bucket of the work size, so later batches on the
-same device skip the search.  The choice only moves work between kernels and
-CTAs: results are identical for every candidate.
+same device skip the search.  The cache carries the identity of the kernels it
+was timed on (build.source_id): choices of another build are dropped, not
+applied.  The choice only moves work between kernels and CTAs: results are
+identical for every candidate.
 """
 from __future__ import annotations
 
@@ -25,6 +27,7 @@ from typing import Callable, Dict, Optional
 import torch
 
 from .binding import BATCH_FUSED, BATCH_MATERIALIZED, team_size
+from .build import source_id
 
 CACHE_DIR = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tune")
 CACHE = os.path.join(CACHE_DIR, "batch_launch.json")
@@ -41,18 +44,21 @@ def candidates(n: int):
 
 
 def _load() -> dict:
+    """The recorded choices of this build's kernels."""
     try:
         with open(CACHE) as f:
-            return json.load(f)
+            d = json.load(f)
     except (OSError, ValueError):
         return {}
+    mine = isinstance(d, dict) and d.get("build") == source_id()
+    return d.get("choices", {}) if mine else {}
 
 
 def _save(d: dict) -> None:
     os.makedirs(CACHE_DIR, exist_ok=True)
     tmp = CACHE + ".tmp"
     with open(tmp, "w") as f:
-        json.dump(d, f, indent=1, sort_keys=True)
+        json.dump({"build": source_id(), "choices": d}, f, indent=1, sort_keys=True)
     os.replace(tmp, CACHE)
 
 
