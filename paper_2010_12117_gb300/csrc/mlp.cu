@@ -7,9 +7,9 @@
 //   W1[64][8] b1[64] W2[64][64] b2[64] W3[2][64] b3[2]   (row = output unit)
 // Loss: mean squared error over the batch and both outputs,
 //   L = 1/(2B) sum_b sum_o (y_bo - t_bo)^2.
-// Kernels: forward (one thread per sample and hidden unit); backward in two
-// deterministic passes - per-sample deltas, then one thread per parameter
-// summing over the batch in a fixed order; Adam.
+// Kernels: forward (one thread per sample and hidden unit, or per sample in
+// large batches); backward in two deterministic passes - per-sample deltas,
+// then one thread per parameter summing over the batch in a fixed order; Adam.
 #include "common.cuh"
 
 namespace {
@@ -26,6 +26,17 @@ static_assert(kParams == POLYDET_MLP_PARAMS, "parameter count");
 // the 64-row step was one CTA with chains of 4096: forward 60 us, deltas 33 us;
 // now 4.6 and 3.1 us, most of it the weights' way from L2.
 constexpr int kSamples = 4;
+
+// Larger batches take a thread per sample (mlp_fwd_rows_kernel,
+// mlp_delta_rows_kernel; the same sums in the same order, so the same bits):
+// they fill the chip by themselves, a CTA's weights serve 128 samples instead
+// of 4, and each multiply-add costs one shared-memory load instead of two.
+// Forward without activations, thread per unit / per sample: 8192 samples 18.0
+// / 18.0 us, 16384 32.7 / 18.2, 65536 123 / 41, 2^20 1928 / 502; with
+// activations (strided stores) 16384 32.9 / 62.3, 65536 124 / 93; backward
+// 16384 861 / 885, 65536 4427 / 4154.
+constexpr int kRowThreads = 128;
+constexpr int kRowsForward = 8192, kRowsTraining = 32768;
 
 __global__ void __launch_bounds__(kSamples *kHid) mlp_fwd_kernel(const float *__restrict__ prm,
                                                                  const float *__restrict__ X, int B,
@@ -59,6 +70,42 @@ __global__ void __launch_bounds__(kSamples *kHid) mlp_fwd_kernel(const float *__
   }
 }
 
+__global__ void __launch_bounds__(kRowThreads)
+    mlp_fwd_rows_kernel(const float *__restrict__ prm, const float *__restrict__ X, int B,
+                        float *__restrict__ Y, float *__restrict__ H) {
+  __shared__ float w[kParams];
+  for (int i = threadIdx.x; i < kParams; i += blockDim.x) w[i] = prm[i];
+  __syncthreads();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= B) return;
+  float x[kIn], h1[kHid];
+#pragma unroll
+  for (int i = 0; i < kIn; ++i) x[i] = X[(int64_t)b * kIn + i];
+#pragma unroll
+  for (int o = 0; o < kHid; ++o) {
+    float s = w[ob1 + o];
+#pragma unroll
+    for (int i = 0; i < kIn; ++i) s = fmaf(w[oW1 + o * kIn + i], x[i], s);
+    h1[o] = fmaxf(s, 0.f);
+  }
+  float y0 = w[ob3], y1 = w[ob3 + 1];
+  for (int o = 0; o < kHid; ++o) {
+    float s = w[ob2 + o];
+#pragma unroll
+    for (int i = 0; i < kHid; ++i) s = fmaf(w[oW2 + o * kHid + i], h1[i], s);
+    const float h2 = fmaxf(s, 0.f);
+    y0 = fmaf(w[oW3 + o], h2, y0);
+    y1 = fmaf(w[oW3 + kHid + o], h2, y1);
+    if (H) H[(int64_t)b * 2 * kHid + kHid + o] = h2;
+  }
+  if (H) {
+#pragma unroll
+    for (int o = 0; o < kHid; ++o) H[(int64_t)b * 2 * kHid + o] = h1[o];
+  }
+  Y[(int64_t)b * kOut] = y0;
+  Y[(int64_t)b * kOut + 1] = y1;
+}
+
 // Per-sample deltas: dY = (y - t) / B; dH2 = W3^T dY * [h2 > 0];
 // dH1 = W2^T dH2 * [h1 > 0].  D[b] = {dY[2], dH2[64], dH1[64]}.  W2's columns
 // are read straight from memory, 32 consecutive words per warp.
@@ -89,6 +136,35 @@ __global__ void __launch_bounds__(kSamples *kHid) mlp_delta_kernel(const float *
 #pragma unroll 32
   for (int o = 0; o < kHid; ++o) s = fmaf(__ldg(prm + oW2 + o * kHid + i), dh2[sl][o], s);
   d[kOut + kHid + i] = h[i] > 0.f ? s : 0.f;
+}
+
+__global__ void __launch_bounds__(kRowThreads)
+    mlp_delta_rows_kernel(const float *__restrict__ prm, const float *__restrict__ T, int B,
+                          const float *__restrict__ Y, const float *__restrict__ H, float *__restrict__ D) {
+  __shared__ float w[kParams];
+  for (int i = threadIdx.x; i < kParams; i += blockDim.x) w[i] = prm[i];
+  __syncthreads();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= B) return;
+  const float *h = H + (int64_t)b * 2 * kHid;
+  float *d = D + (int64_t)b * (kOut + 2 * kHid);
+  const float dy0 = (Y[(int64_t)b * kOut] - T[(int64_t)b * kOut]) / (float)B;
+  const float dy1 = (Y[(int64_t)b * kOut + 1] - T[(int64_t)b * kOut + 1]) / (float)B;
+  d[0] = dy0;
+  d[1] = dy1;
+  float dh2[kHid];
+#pragma unroll
+  for (int o = 0; o < kHid; ++o) {
+    const float g = w[oW3 + o] * dy0 + w[oW3 + kHid + o] * dy1;
+    dh2[o] = h[kHid + o] > 0.f ? g : 0.f;
+    d[kOut + o] = dh2[o];
+  }
+  for (int i = 0; i < kHid; ++i) {
+    float s = 0.f;
+#pragma unroll
+    for (int o = 0; o < kHid; ++o) s = fmaf(w[oW2 + o * kHid + i], dh2[o], s);
+    d[kOut + kHid + i] = h[i] > 0.f ? s : 0.f;
+  }
 }
 
 // One thread per parameter (and one more for the loss): sums over the batch
@@ -149,8 +225,12 @@ __global__ void mlp_adam_kernel(float *__restrict__ prm, const float *__restrict
 extern "C" int polydet_mlp_forward(const float *params, const float *x, int batch, float *y,
                                    float *act_ws, void *stream) {
   if (!params || !x || !y || batch < 1) return POLYDET_EINVAL;
-  mlp_fwd_kernel<<<(batch + kSamples - 1) / kSamples, kSamples * kHid, 0, (cudaStream_t)stream>>>(params, x, batch,
-                                                                                               y, act_ws);
+  cudaStream_t st = (cudaStream_t)stream;
+  if (batch > (act_ws ? kRowsTraining : kRowsForward))
+    mlp_fwd_rows_kernel<<<(unsigned)(((int64_t)batch + kRowThreads - 1) / kRowThreads), kRowThreads, 0, st>>>(
+        params, x, batch, y, act_ws);
+  else
+    mlp_fwd_kernel<<<(batch + kSamples - 1) / kSamples, kSamples * kHid, 0, st>>>(params, x, batch, y, act_ws);
   PD_CUDA(cudaGetLastError());
   return POLYDET_OK;
 }
@@ -162,8 +242,12 @@ extern "C" int polydet_mlp_backward(const float *params, const float *x, const f
     return POLYDET_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   const int th = 128;
-  mlp_delta_kernel<<<(batch + kSamples - 1) / kSamples, kSamples * kHid, 0, st>>>(params, target, batch, y, act_ws,
-                                                                                  delta_ws);
+  if (batch > kRowsTraining)
+    mlp_delta_rows_kernel<<<(unsigned)(((int64_t)batch + kRowThreads - 1) / kRowThreads), kRowThreads, 0, st>>>(
+        params, target, batch, y, act_ws, delta_ws);
+  else
+    mlp_delta_kernel<<<(batch + kSamples - 1) / kSamples, kSamples * kHid, 0, st>>>(params, target, batch, y,
+                                                                                   act_ws, delta_ws);
   PD_CUDA(cudaGetLastError());
   mlp_grad_kernel<<<(kParams + 1 + th - 1) / th, th, 0, st>>>(x, target, batch, y, act_ws, delta_ws,
                                                               grads, loss);
