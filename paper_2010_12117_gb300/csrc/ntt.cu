@@ -336,20 +336,31 @@ struct CiArgs {
   int tab_len;          // words per prime
 };
 
-// sum_{j<len} x[j] y[j s] / R mod p (x from global memory, y from shared
-// memory with stride s): four products per REDC (redc4: 4 p^2 < p 2^32 for
-// any p < 2^31; fewer in the last one).
+// A table word from shared memory (TAB) or global memory.
+template <bool TAB>
+PD_D uint32_t ci_ld(const uint32_t *x) {
+  if constexpr (TAB)
+    return *x;
+  else
+    return __ldg(x);
+}
+
+// sum_{j<len} x[j] y[j s] / R mod p (x a table, y in shared memory with stride
+// s): four products per REDC (redc4: 4 p^2 < p 2^32 for any p < 2^31; fewer in
+// the last one).
+template <bool TAB>
 PD_D uint32_t dot_strided(const uint32_t *x, const uint32_t *y, int s, int len, uint32_t p, uint32_t pinv) {
   uint32_t acc = 0u;
   int j = 0;
   for (; j + 3 < len; j += 4)
     acc = addm(acc,
-               redc4((uint64_t)__ldg(x + j) * y[j * s] + (uint64_t)__ldg(x + j + 1) * y[(j + 1) * s] +
-                         (uint64_t)__ldg(x + j + 2) * y[(j + 2) * s] + (uint64_t)__ldg(x + j + 3) * y[(j + 3) * s],
+               redc4((uint64_t)ci_ld<TAB>(x + j) * y[j * s] + (uint64_t)ci_ld<TAB>(x + j + 1) * y[(j + 1) * s] +
+                         (uint64_t)ci_ld<TAB>(x + j + 2) * y[(j + 2) * s] +
+                         (uint64_t)ci_ld<TAB>(x + j + 3) * y[(j + 3) * s],
                      p, pinv),
                p);
   uint64_t t = 0u;
-  for (; j < len; ++j) t += (uint64_t)__ldg(x + j) * y[j * s];
+  for (; j < len; ++j) t += (uint64_t)ci_ld<TAB>(x + j) * y[j * s];
   return addm(acc, redc4(t, p, pinv), p);
 }
 
@@ -382,11 +393,19 @@ PD_D void small_dft(uint32_t (&x)[L], const uint32_t *rk, uint32_t p, uint32_t p
 constexpr int kCiU = 4;  // coefficients per thread and column (one 16-byte table load)
 
 // U: coefficients per thread, kCiU, or 1 where a pass is too small to fill the
-// chip and its time is one thread's chain of products (24 x 24 univariate, two
-// primes: interpolation + CRT 7.1 us with four, 6.0 with one).
-template <int L, int U>
-__global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
-  extern __shared__ uint32_t sm[];
+// chip and its time is one thread's chain of products.
+// TAB (U == 1): the tables staged in shared memory, one trip to L2 for all of
+// them instead of one per four products of that chain; chains of more than two
+// such steps, tables of at most 16 KB (longer ones pass through 1024 threads
+// that cover the trips for each other).  One prime, microseconds, tables in
+// global memory and 256 threads / now: 24 x 24 univariate, degree 7 (169
+// nodes) 5.9 / 5.1; 32 x 32, degree 3 6.0 / 4.6; 19 x 19, degree 200 (3801
+// nodes) 380 / 193; 8 x 8, degrees 5 and 200 150 / 48; but 3 x 3, degree 1
+// (chains of one step) 2.3 / 2.6 staged.
+constexpr int kCiSmallThreads = 1024, kCiTabWords = 4096;
+template <int L, int U, bool TAB>
+__global__ void __launch_bounds__(U == 1 ? kCiSmallThreads : 256) cinterp_kernel(CiArgs a) {
+  extern __shared__ __align__(16) uint32_t sm[];
   const int q = a.prime_lo + blockIdx.z;
   const ModP md = a.mod[q];
   const uint32_t p = md.p, pinv = md.pinv;
@@ -397,8 +416,8 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
   const uint32_t *in = a.in + (int64_t)blockIdx.z * a.in_prime_stride;
   uint32_t *out = a.out + (int64_t)blockIdx.z * a.out_prime_stride;
   const CiTab T(m, L);
-  const uint32_t *tab = a.tab + (size_t)q * a.tab_len;
-  uint32_t *Qv = sm;                                 // [L][JJ][Ct] Q_r(z_j), then lambda_r
+  const uint32_t *gtab = a.tab + (size_t)q * a.tab_len, *tab = TAB ? sm : gtab;
+  uint32_t *Qv = sm + (TAB ? T.words : 0);           // [L][JJ][Ct] Q_r(z_j), then lambda_r
   uint32_t *Es = Qv + (size_t)L * JJ * Ct;           // [L][Ct] E_r (s > 0)
   uint32_t *Y = Es + (s > 0 ? (size_t)L * Ct : 0);   // [Ct][mp] node values, then coefficients (rows)
   const int mp = m | 1;                              // odd: lanes of different columns in different banks
@@ -414,6 +433,9 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
   // a thread keeps its column through the phases (blockDim is a multiple of Ct)
   const int c = tid & (Ct - 1), jstep = bd >> logCt;
 
+  if constexpr (TAB)  // read from step 2 on; the parts are multiples of 16 bytes
+    for (int i = tid; i < T.words / 4; i += bd)
+      reinterpret_cast<uint4 *>(sm)[i] = __ldg(reinterpret_cast<const uint4 *>(gtab) + i);
   if (a.rows) {
     const uint32_t *src = in + col0 * m;
     for (int k = tid >> 5; k < ncol; k += bd >> 5)
@@ -426,13 +448,13 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
   // 1. inverse DFT of each whole coset, twisted
   {
     const uint32_t *sj = src + (int64_t)(tid >> logCt) * L * sstep;
-    const uint32_t *tw = tab + T.tw1 + (tid >> logCt) * L;
+    const uint32_t *tw = gtab + T.tw1 + (tid >> logCt) * L;
     uint32_t *qj = Qv + ((tid >> logCt) << logCt) + c;
     for (int j = tid >> logCt; j < Jf; j += jstep) {
       uint32_t x[L];
 #pragma unroll
       for (int t = 0; t < L; ++t) x[t] = c < ncol ? sj[t * sstep] : 0u;
-      small_dft<L>(x, tab + T.rk, p, pinv);
+      small_dft<L>(x, gtab + T.rk, p, pinv);
 #pragma unroll
       for (int r = 0; r < L; ++r) qj[(r * JJ) << logCt] = mmul(x[r], __ldg(tw + r), p, pinv);
       sj += (int64_t)jstep * L * sstep;
@@ -440,17 +462,31 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
       qj += jstep << logCt;
     }
   }
+  // the last coset's values: where a chain bounds the pass and there are
+  // several, loaded ahead and all at once
+  constexpr bool AHEAD = U == 1 && L > 2;
+  uint32_t last[L];
+  if constexpr (AHEAD) {
+#pragma unroll
+    for (int t = 0; t + 1 < L; ++t) last[t] = (t < s && c < ncol) ? src[(Jf * L + t) * sstep] : 0u;
+  }
   __syncthreads();
   if (s > 0) {  // 2. the last coset
     for (int r = tid >> logCt; r < L; r += jstep)
-      Es[(r << logCt) + c] = dot_strided(tab + T.ell, Qv + ((r * JJ) << logCt) + c, Ct, Jf, p, pinv);
+      Es[(r << logCt) + c] = dot_strided<TAB>(tab + T.ell, Qv + ((r * JJ) << logCt) + c, Ct, Jf, p, pinv);
     __syncthreads();
     for (int r = tid >> logCt; r < L; r += jstep) {
       uint32_t lam = 0u;
       if (r < s && c < ncol) {
-        lam = dot_strided(tab + T.nx + r * L, Es + c, Ct, L, p, pinv);
-        for (int t = 0; t < s; ++t)
-          lam = addm(lam, mmul(__ldg(tab + T.bm + r * s + t), src[(Jf * L + t) * sstep], p, pinv), p);
+        lam = dot_strided<TAB>(tab + T.nx + r * L, Es + c, Ct, L, p, pinv);
+        if constexpr (AHEAD) {
+#pragma unroll
+          for (int t = 0; t + 1 < L; ++t)
+            if (t < s) lam = addm(lam, mmul(ci_ld<TAB>(tab + T.bm + r * s + t), last[t], p, pinv), p);
+        } else {
+          for (int t = 0; t < s; ++t)
+            lam = addm(lam, mmul(ci_ld<TAB>(tab + T.bm + r * s + t), src[(Jf * L + t) * sstep], p, pinv), p);
+        }
       }
       Qv[((r * JJ + Jf) << logCt) + c] = lam;
     }
@@ -484,7 +520,7 @@ __global__ void __launch_bounds__(256) cinterp_kernel(CiArgs a) {
           const uint4 v4 = __ldg(reinterpret_cast<const uint4 *>(V + k * vstep));
           v[0] = v4.x, v[1] = v4.y, v[2] = v4.z, v[3] = v4.w;
         } else {
-          v[0] = __ldg(V + k * vstep);
+          v[0] = ci_ld<TAB>(V + k * vstep);
         }
         const uint32_t y0 = y[k << logCt], y1 = y[(k << logCt) + half];
 #pragma unroll
@@ -551,15 +587,19 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
   PD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   static PdPerDevice attr;
   const int arc = pd_once_per_device(attr, [] {
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<1, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<2, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<4, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    PD_CUDA(cudaFuncSetAttribute(cinterp_kernel<8, kCiU>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-    return POLYDET_OK;
+    int rc = POLYDET_OK;
+    auto allow = [&](auto kern) {
+      if (rc == POLYDET_OK)
+        rc = [&] {
+          PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+          return POLYDET_OK;
+        }();
+    };
+    allow(cinterp_kernel<1, kCiU, false>), allow(cinterp_kernel<1, 1, false>), allow(cinterp_kernel<1, 1, true>);
+    allow(cinterp_kernel<2, kCiU, false>), allow(cinterp_kernel<2, 1, false>), allow(cinterp_kernel<2, 1, true>);
+    allow(cinterp_kernel<4, kCiU, false>), allow(cinterp_kernel<4, 1, false>), allow(cinterp_kernel<4, 1, true>);
+    allow(cinterp_kernel<8, kCiU, false>), allow(cinterp_kernel<8, 1, false>), allow(cinterp_kernel<8, 1, true>);
+    return rc;
   });
   if (arc) return arc;
   const uint32_t *cur = detvals;
@@ -584,20 +624,28 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
     // grid still spreads over the SMs (two CTAs each) and every CTA's
     // phases, which run one after another, are short
     while (ct > 4 && (ncols + ct - 1) / ct * np < 2 * sms) ct >>= 1;
-    const size_t smem = cinterp_words(a.m, L, ct, a.rows) * sizeof(uint32_t);
-    if (smem > kMaxSmem) return POLYDET_EINVAL;
-    a.Ct = ct;
-    a.logCt = ilog2(ct);
+    // fewer columns still, while every CTA has an SM to itself
+    while (ct > 2 && (ncols + ct / 2 - 1) / (ct / 2) * np <= sms) ct >>= 1;
+    const int64_t ctas = (ncols + ct - 1) / ct * np;
+    int items = std::max(1, (a.Jf + kCiU - 1) / kCiU) * L * (ct / 2);
+    const bool small = ctas * items < 256 * sms;
+    if (small) items = std::max(1, a.Jf) * L * (ct / 2);
     // threads: a multiple of the columns, no more than step 3 has items for.
     // Small CTAs, so that those of an SM are in different phases (73^3 nodes,
     // 18 primes: 172 us with 128 threads, 180 with 192, 207 with 512; 64
     // columns and 320 threads 186), larger ones where the grid is short of
     // four CTAs per SM (193^2 nodes, 24 primes: 34.8 us with 256, 36.9 with 128)
-    const int64_t ctas = (ncols + ct - 1) / ct * np;
-    int items = std::max(1, (a.Jf + kCiU - 1) / kCiU) * L * (ct / 2);
-    const bool small = ctas * items < 256 * sms;
-    if (small) items = std::max(1, a.Jf) * L * (ct / 2);
-    const int th = std::min((items + 63) / 64 * 64, ctas >= 4 * sms ? 128 : 256);
+    // and the largest where it is short of one
+    const int most = ctas >= 4 * sms ? 128 : small && ctas <= sms ? kCiSmallThreads : 256;
+    const int th = std::min((items + 63) / 64 * 64, most);
+    size_t smem = cinterp_words(a.m, L, ct, a.rows) * sizeof(uint32_t);
+    const int tab_words = CiTab(a.m, L).words;
+    const bool staged =
+        small && a.Jf > 8 && tab_words <= kCiTabWords && smem + tab_words * sizeof(uint32_t) <= kMaxSmem;
+    if (staged) smem += tab_words * sizeof(uint32_t);
+    if (smem > kMaxSmem) return POLYDET_EINVAL;
+    a.Ct = ct;
+    a.logCt = ilog2(ct);
     a.in = cur;
     a.in_prime_stride = cur_prime;
     if (v == 0) {
@@ -612,20 +660,20 @@ static int interp_nodes(polydet_plan_t pl, const uint32_t *detvals, int lo, int 
     a.tab = pl->d_itab + pl->itab_off[v];
     a.tab_len = pl->itab_len;
     dim3 grid((unsigned)((ncols + ct - 1) / ct), 1, (unsigned)np);
-    if (small) {
-      switch (L) {
-        case 1: cinterp_kernel<1, 1><<<grid, th, smem, st>>>(a); break;
-        case 2: cinterp_kernel<2, 1><<<grid, th, smem, st>>>(a); break;
-        case 4: cinterp_kernel<4, 1><<<grid, th, smem, st>>>(a); break;
-        default: cinterp_kernel<8, 1><<<grid, th, smem, st>>>(a); break;
-      }
-    } else {
-      switch (L) {
-        case 1: cinterp_kernel<1, kCiU><<<grid, th, smem, st>>>(a); break;
-        case 2: cinterp_kernel<2, kCiU><<<grid, th, smem, st>>>(a); break;
-        case 4: cinterp_kernel<4, kCiU><<<grid, th, smem, st>>>(a); break;
-        default: cinterp_kernel<8, kCiU><<<grid, th, smem, st>>>(a); break;
-      }
+    auto launch = [&](auto len) {
+      constexpr int LL = decltype(len)::value;
+      if (staged)
+        cinterp_kernel<LL, 1, true><<<grid, th, smem, st>>>(a);
+      else if (small)
+        cinterp_kernel<LL, 1, false><<<grid, th, smem, st>>>(a);
+      else
+        cinterp_kernel<LL, kCiU, false><<<grid, th, smem, st>>>(a);
+    };
+    switch (L) {
+      case 1: launch(std::integral_constant<int, 1>()); break;
+      case 2: launch(std::integral_constant<int, 2>()); break;
+      case 4: launch(std::integral_constant<int, 4>()); break;
+      default: launch(std::integral_constant<int, 8>()); break;
     }
     PD_CUDA(cudaGetLastError());
     cur = a.out;
