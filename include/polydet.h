@@ -423,11 +423,18 @@ int polydet_team_size(int n);
 /* Columns of the pivot blocks the condensation kernels of order n eliminate
  * by (2 or 3); POLYDET_EINVAL outside 1..32.  Host only. */
 int polydet_condense_steps(int n);
-/* Columns the condensation kernels of order n eliminate at a time: 2 or 3, or
- * 4 where two 2 x 2 pivot blocks are applied together (the instruction mix,
- * and so the integer-pipe ceiling, depends on it); POLYDET_EINVAL outside
- * 1..32.  Host only. */
+/* Columns the condensation kernel of large launches of order n eliminates at a
+ * time: 2 or 3, or 4 where two 2 x 2 pivot blocks are applied together (the
+ * instruction mix, and so the integer-pipe ceiling, depends on it);
+ * POLYDET_EINVAL outside 1..32.  Host only. */
 int polydet_condense_columns(int n);
+/* The condensation kernel a launch of `matrices` matrices of order n (nodes x
+ * primes, `prime` the largest) takes: launch[0] lanes that share a matrix,
+ * launch[1] columns eliminated at a time (2 to 4), launch[2] CTAs per SM it is
+ * compiled for, launch[3] threads per CTA; small launches and primes above
+ * 1865126253 have kernels of their own at some orders.  POLYDET_EINVAL for n
+ * outside 1..32 or matrices < 1.  Host only. */
+int polydet_condense_launch(int n, long long matrices, unsigned prime, int32_t launch[4]);
 
 /* Stage 1 of a batch (Sec. 3.1): every variable but the last (fused orders)
  * or but the first (materialized orders); all orders (n = 0 in

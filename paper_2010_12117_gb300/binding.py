@@ -126,6 +126,7 @@ SIGNATURES = {
                                      ctypes.POINTER(ctypes.c_double)]),
     "polydet_condense_steps": (_I, [_I]),
     "polydet_condense_columns": (_I, [_I]),
+    "polydet_condense_launch": (_I, [_I, ctypes.c_longlong, ctypes.c_uint32, _PI32]),
     "polydet_last_error": (ctypes.c_char_p, []),
 }
 
@@ -616,11 +617,19 @@ def condense_steps(n: int) -> int:
 
 
 def condense_columns(n: int) -> int:
-    """Columns the condensation kernels of order n eliminate at a time (2, 3 or 4)."""
+    """Columns the condensation kernel of large launches of order n eliminates at a time (2, 3 or 4)."""
     t = lib().polydet_condense_columns(int(n))
     if t < 1:
         _check(t, "polydet_condense_columns")
     return t
+
+
+def condense_launch(n: int, matrices: int, prime: int = 0) -> tuple:
+    """(lanes per matrix, columns at a time, CTAs per SM, threads per CTA) of the kernel that condenses
+    ``matrices`` matrices of order n, ``prime`` the largest of the launch."""
+    out = (ctypes.c_int32 * 4)()
+    _check(lib().polydet_condense_launch(int(n), int(matrices), int(prime), out), "polydet_condense_launch")
+    return tuple(out)
 
 
 def limbs_to_ints(limbs: np.ndarray, W: int) -> List[int]:

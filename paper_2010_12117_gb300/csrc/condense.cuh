@@ -490,9 +490,10 @@ __global__ void __launch_bounds__(TH, MINB) condense_kernel(const uint32_t *__re
   else
     sink = {&s_piv[0][team], S, t == 0, false};
   fast_pass<NN, T, STEP, 0>(a, p, pinv, sink);
-  // larger primes (only plans of more than 67 reach them) redo every matrix
-  // with the pivoting elimination (the fast pass is not skipped: a branch
-  // around it costs the common case its register allocation)
+  // larger primes (only plans of more than 67 reach them, and not at the orders
+  // of cond_wide that take triples for them) redo every matrix with the
+  // pivoting elimination (the fast pass is not skipped: a branch around it
+  // costs the common case its register allocation)
   if (step_folds3(STEP)) sink.zero |= p > PD_FOLD3_MAX;
   const bool redo = __any_sync(PD_FULL, sink.zero);  // some matrix of this warp met a zero pivot
   uint2 qd = make_uint2(0u, 0u);
@@ -533,11 +534,11 @@ static inline size_t condense_reserve_bytes(int ctas) {
   return (size_t)per_sm / (size_t)(ctas + 1) + 1024;
 }
 
-template <int NN, bool FEW>
+template <int NN, int PICK>
 static int condense_launch(const polydet_plan_s *pl, const uint32_t *evals, EvLayout lay, int64_t G,
                            int64_t det_stride, int prime_lo, int nprimes, uint32_t *detvals,
                            int ctas_per_sm, cudaStream_t st) {
-  constexpr CondCfg cfg = FEW ? cond_few(NN) : kCond[NN];
+  constexpr CondCfg cfg = cond_cfg(NN, PICK);
   constexpr int T = cfg.team, threads = cfg.threads;
   auto kern = condense_kernel<NN, T, cfg.step, cfg.ctas, threads, cfg.lane_pivots>;
   const size_t reserve = condense_reserve_bytes(ctas_per_sm);
@@ -564,10 +565,18 @@ static int condense_dispatch(const polydet_plan_s *pl, const uint32_t *evals, Ev
                              int64_t G, int64_t det_stride, int prime_lo, int nprimes,
                              uint32_t *detvals, int ctas_per_sm, cudaStream_t st) {
   if (pl->n == NN) {
+    bool wide = false;
+    for (int q = prime_lo; q < prime_lo + nprimes; ++q) wide |= pl->primes[q] > PD_FOLD3_MAX;
+    const int pick = cond_pick(NN, G * nprimes, wide);
+    auto launch = [&](auto kind) {
+      return condense_launch<NN, decltype(kind)::value>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals,
+                                                        ctas_per_sm, st);
+    };
+    if constexpr (cond_has_wide(NN))
+      if (pick == 2) return launch(std::integral_constant<int, 2>());
     if constexpr (!cond_same(cond_few(NN), kCond[NN]))
-      if (G * nprimes <= kCondFew)
-        return condense_launch<NN, true>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
-    return condense_launch<NN, false>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
+      if (pick == 1) return launch(std::integral_constant<int, 1>());
+    return launch(std::integral_constant<int, 0>());
   }
   if constexpr (NN < HI)
     return condense_dispatch<NN + 1, HI>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals,

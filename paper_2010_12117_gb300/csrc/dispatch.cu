@@ -52,7 +52,17 @@ int pd_launch_condense_nodes(const polydet_plan_s *pl, const uint32_t *evals, Ev
                              int64_t det_stride, int prime_lo, int nprimes, uint32_t *detvals,
                              cudaStream_t st, int ctas_per_sm) {
   const int n = pl->n;
-  if (n < 1 || G < 1) return POLYDET_EINVAL;
+  if (n < 1 || n > POLYDET_MAX_N || G < 1) return POLYDET_EINVAL;
+  // primes above PD_FOLD3_MAX come last (prime table)
+  int low = 0;
+  while (low < nprimes && pl->primes[prime_lo + low] <= PD_FOLD3_MAX) ++low;
+  if (low < nprimes && cond_has_wide(n) && G * low >= kCondSplit) {
+    const int rc = pd_launch_condense_nodes(pl, evals, lay, G, det_stride, prime_lo, low, detvals, st, ctas_per_sm);
+    if (rc) return rc;
+    return pd_launch_condense_nodes(pl, evals + (int64_t)low * pl->nent * lay.entry, lay, G, det_stride,
+                                    prime_lo + low, nprimes - low, detvals + (int64_t)low * det_stride, st,
+                                    ctas_per_sm);
+  }
   if (n <= 6) return pd_condense_from_1(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
   if (n <= 10) return pd_condense_from_7(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
   if (n <= 12) return pd_condense_from_11(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals, ctas_per_sm, st);
@@ -100,6 +110,16 @@ extern "C" int polydet_team_size(int n) {
 
 extern "C" int polydet_condense_steps(int n) {
   return (n >= 1 && n <= POLYDET_MAX_N) ? (kCond[n].step == 3 ? 3 : 2) : POLYDET_EINVAL;
+}
+
+extern "C" int polydet_condense_launch(int n, long long matrices, unsigned prime, int32_t launch[4]) {
+  if (n < 1 || n > POLYDET_MAX_N || matrices < 1 || !launch) return POLYDET_EINVAL;
+  const CondCfg c = cond_cfg(n, cond_pick(n, matrices, prime > PD_FOLD3_MAX));
+  launch[0] = c.team;
+  launch[1] = c.step;
+  launch[2] = c.ctas;
+  launch[3] = c.threads;
+  return POLYDET_OK;
 }
 
 extern "C" int polydet_condense_columns(int n) {

@@ -60,10 +60,41 @@ constexpr CondCfg cond_few(int n) {
          : n == 30           ? CondCfg{8, 2, 3, 128, true}
                              : kCond[n];
 }
+
+// Launches that hold a prime above PD_FOLD3_MAX, which pairs and quads can only
+// redo one step at a time.  Orders whose triples come near the quads (or win in
+// small launches) take triples, which any prime passes; 25 to 28, whose large
+// launches have four lanes, redo with eight.  The others stay with their
+// pairs or quads and redo.  30000 matrices and three such primes, microseconds, redone
+// quads / this choice: order 10 28.2 / 13.5, 15 86 / 37, 17 144 / 56, 18 189 /
+// 73, 19 180 / 77, 21 254 / 104, 23 439 / 128, 26 707 / 527, 28 1182 / 672.
+constexpr CondCfg cond_wide(int n) {
+  return n == 10              ? CondCfg{1, 3, 4, 128, true}
+         : n == 15 || n == 17 ? CondCfg{2, 3, 4, 128, true}
+         : n == 18 || n == 19 ? CondCfg{2, 3, 3, 128, true}
+         : n == 21            ? CondCfg{4, 3, 2, 256, true}
+         : n == 23            ? CondCfg{4, 3, 4, 128, true}
+         : n >= 25 && n <= 28 ? CondCfg{8, 4, 4, 128, true}
+                              : kCond[n];
+}
+
 constexpr bool cond_same(CondCfg a, CondCfg b) {
   return a.team == b.team && a.step == b.step && a.ctas == b.ctas && a.threads == b.threads &&
          a.lane_pivots == b.lane_pivots;
 }
+
+// The kernel of a launch of `matrices` matrices of order n, `wide` where it
+// holds a prime above PD_FOLD3_MAX: 0 kCond, 1 cond_few, 2 cond_wide.
+constexpr bool cond_has_wide(int n) { return !cond_same(cond_wide(n), kCond[n]); }
+constexpr int cond_pick(int n, int64_t matrices, bool wide) {
+  return wide && cond_has_wide(n) ? 2 : !cond_same(cond_few(n), kCond[n]) && matrices <= kCondFew ? 1 : 0;
+}
+constexpr CondCfg cond_cfg(int n, int pick) { return pick == 2 ? cond_wide(n) : pick == 1 ? cond_few(n) : kCond[n]; }
+
+// A range of primes that straddles PD_FOLD3_MAX is launched in two parts where
+// the lower part is long enough for its kernel's lead (5 % at order 21) to pay
+// for the second launch's last wave (about half a wave): a dozen waves.
+constexpr int64_t kCondSplit = 1 << 18;
 
 // The fused kernels (fused.cuh): lanes per matrix and columns per step.  One
 // lane while the whole matrix fits in registers (n <= 12), then 2, 4 and 8:
