@@ -567,15 +567,18 @@ static int condense_dispatch(const polydet_plan_s *pl, const uint32_t *evals, Ev
   if (pl->n == NN) {
     bool wide = false;
     for (int q = prime_lo; q < prime_lo + nprimes; ++q) wide |= pl->primes[q] > PD_FOLD3_MAX;
-    const int pick = cond_pick(NN, G * nprimes, wide);
+    const int pick = cond_canonical(NN, cond_pick(NN, G * nprimes, wide));
     auto launch = [&](auto kind) {
       return condense_launch<NN, decltype(kind)::value>(pl, evals, lay, G, det_stride, prime_lo, nprimes, detvals,
                                                         ctas_per_sm, st);
     };
-    if constexpr (cond_has_wide(NN))
-      if (pick == 2) return launch(std::integral_constant<int, 2>());
-    if constexpr (!cond_same(cond_few(NN), kCond[NN]))
+    if constexpr (cond_canonical(NN, 1) == 1)
       if (pick == 1) return launch(std::integral_constant<int, 1>());
+    if constexpr (cond_canonical(NN, 2) == 2)
+      if (pick == 2) return launch(std::integral_constant<int, 2>());
+    if constexpr (cond_canonical(NN, 3) == 3)
+      if (pick == 3) return launch(std::integral_constant<int, 3>());
+    static_assert(kPickWide == 3, "one branch per choice");
     return launch(std::integral_constant<int, 0>());
   }
   if constexpr (NN < HI)

@@ -50,3 +50,37 @@ def test_every_choice_is_a_launchable_kernel(binding):
     for bad in (0, 33):
         with pytest.raises(binding.PolydetError):
             binding.condense_columns(bad)
+
+
+SMALL = {8: (0, 65536), 9: (0, 32768), 10: (0, 131072), 13: (0, 19456), 16: (0, 65536), 19: (14593, 19456),
+         23: (0, 14592), 25: (0, 7296), 26: (0, 7296), 27: (0, 7296), 28: (0, 7296), 31: (0, 21888), 32: (0, 65536)}
+
+
+@pytest.mark.parametrize("n", range(1, 33))
+def test_small_launches_have_their_own_range(binding, n):
+    """Orders whose small launches take another kernel do so inside their range and nowhere else."""
+    large = binding.condense_launch(n, 10 ** 9)
+    lo, hi = SMALL.get(n, (0, -1))
+    end = 9728 if n in (25, 28) else hi  # a second choice follows the first
+    for m in (1, 100, 4800, 7296, 7297, 9728, 9729, 14592, 14593, 19300, 19456, 19457, 21888, 21889, 32768, 32769,
+              65536, 65537, 131072, 131073, 200_000):
+        own = binding.condense_launch(n, m)
+        if lo <= m <= end:
+            assert n == 31 or own != large, (n, m)  # order 31 differs in where the pivots are folded
+        else:
+            assert own == large, (n, m)
+
+
+@pytest.mark.parametrize("n", [16, 23, 26, 32])
+@pytest.mark.parametrize("matrices", [30, 100, 1200, 2400, 4800, 7200])
+def test_launches_below_a_wave_take_small_ctas(binding, n, matrices):
+    """Three CTAs of 128 threads per SM: short of a wave, larger CTAs leave some SMs with twice the warps of others,
+    and four CTAs have fewer registers per thread."""
+    assert binding.condense_launch(n, matrices)[2:] == (3, 128)
+
+
+def test_large_primes_do_not_redo_what_triples_pass(binding):
+    for n in range(1, 33):
+        if binding.condense_columns(n) == 3:
+            for matrices in SIZES:
+                assert binding.condense_launch(n, matrices, FOLD3_MAX + 1)[1] == 3, (n, matrices)

@@ -72,3 +72,21 @@ def test_primes_on_both_sides_of_the_fold_limit(n, matrices):
 def test_long_ranges_split_at_the_fold_limit(n):
     """More than 2^18 matrices below the limit: the part above it is a launch of its own."""
     _check(n, 270_000, 2, 69, 66)
+
+
+def _launches(n, prime):
+    """(smallest, largest) launch up to 140000 matrices of every kernel of order n."""
+    from paper_2010_12117_gb300 import binding
+    sizes = [97, 7000, 7297, 9700, 9729, 14500, 14593, 19400, 19457, 21800, 21889, 32700, 32769, 65000, 65537,
+             131000, 131073, 140000]
+    kernels = {}
+    for m in sizes:
+        kernels.setdefault(binding.condense_launch(n, m, prime), []).append(m)
+    return sorted({m for ms in kernels.values() for m in (ms[0], next((x for x in ms[1:] if x > 21900), ms[-1]))})
+
+
+@pytest.mark.parametrize("n", range(1, 33))
+def test_every_kernel_of_an_order(n):
+    """Each kernel the launch rule names for order n, in its smallest launch and one of several waves."""
+    for matrices in _launches(n, 0):
+        _check(n, matrices, 1, 1 + n % 3, n % 3)
