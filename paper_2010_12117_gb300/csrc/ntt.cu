@@ -119,29 +119,60 @@ static int ilog2(int64_t x) {
   return l;
 }
 
+// How a pass is split over threads: columns per thread, threads per CTA, a
+// flattened grid (TxArgs::flat_items), and the CTAs an SM may hold (0: any).
+struct DirectShape {
+  int cpt, threads;
+  bool flat;
+  int ctas;
+};
+
+// The dynamic shared memory that keeps a CTA's SM to `ctas` of them.
+static size_t direct_reserve_bytes(int ctas) {
+  if (ctas <= 0) return 0;
+  int per_sm = 0, dev = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  // static twiddles and the 1 KB the system keeps per CTA count as well
+  return (size_t)per_sm / (ctas + 1) + 256 - kDirectTwSmem * sizeof(uint2) - 1024;
+}
+
 template <int CPT, class Off, bool FLAT>
-static int launch_direct_as(const TxArgs &a, dim3 grid, cudaStream_t st) {
-  constexpr int TH = kDirectThreads;
+static int launch_direct_as(const TxArgs &a, dim3 grid, const DirectShape &s, cudaStream_t st) {
+  const size_t reserve = direct_reserve_bytes(s.ctas);
+  auto launch = [&](auto lin) {
+    auto kern = coltx_direct_kernel<decltype(lin)::value, CPT, Off, FLAT>;
+    if (reserve) {
+      static PdPerDevice attr;
+      const int rc = pd_once_per_device(attr, [&] {
+        PD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 120 * 1024));
+        return POLYDET_OK;
+      });
+      if (rc) return rc;
+    }
+    kern<<<grid, s.threads, reserve, st>>>(a);
+    PD_CUDA(cudaGetLastError());
+    return POLYDET_OK;
+  };
   switch (a.Lin) {
-    case 1: coltx_direct_kernel<1, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    case 2: coltx_direct_kernel<2, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    case 3: coltx_direct_kernel<3, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    case 4: coltx_direct_kernel<4, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    case 5: coltx_direct_kernel<5, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    case 6: coltx_direct_kernel<6, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    case 7: coltx_direct_kernel<7, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
-    default: coltx_direct_kernel<8, CPT, Off, FLAT><<<grid, TH, 0, st>>>(a); break;
+    case 1: return launch(std::integral_constant<int, 1>());
+    case 2: return launch(std::integral_constant<int, 2>());
+    case 3: return launch(std::integral_constant<int, 3>());
+    case 4: return launch(std::integral_constant<int, 4>());
+    case 5: return launch(std::integral_constant<int, 5>());
+    case 6: return launch(std::integral_constant<int, 6>());
+    case 7: return launch(std::integral_constant<int, 7>());
+    default: return launch(std::integral_constant<int, 8>());
   }
-  PD_CUDA(cudaGetLastError());
-  return POLYDET_OK;
 }
 
 template <int CPT>
-static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes, cudaStream_t st) {
-  constexpr int TH = kDirectThreads;
-  dim3 grid((unsigned)((ncols + TH * CPT - 1) / (TH * CPT)), (unsigned)items, (unsigned)nprimes);
+static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes, const DirectShape &s,
+                         cudaStream_t st) {
+  const int64_t per = (int64_t)s.threads * CPT;
+  dim3 grid((unsigned)((ncols + per - 1) / per), (unsigned)items, (unsigned)nprimes);
   if (a.flat_items)
-    grid = dim3((unsigned)((ncols * items * a.flat_groups + TH - 1) / TH), 1u, (unsigned)nprimes);
+    grid = dim3((unsigned)((ncols * items * a.flat_groups + s.threads - 1) / s.threads), 1u, (unsigned)nprimes);
   // 32-bit byte offsets where all the output a CTA's base pointer covers lies
   // within 4 GB of it (rows the kernel steps over past the last one included)
   const int64_t rows = (int64_t)a.N + 8;
@@ -150,15 +181,81 @@ static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes,
     span = (rows * (a.B / a.il_L) + 1) * a.il_n2 * a.il_Lp;
   else
     span = (a.flat_items ? (int64_t)items * a.out_item_stride : 0) +
-           a.A * rows * (a.out_row ? a.out_row : a.B) + TH * CPT;
+           a.A * rows * (a.out_row ? a.out_row : a.B) + per;
   const bool near = span < ((int64_t)1 << 30);
   if constexpr (CPT == 1) {
     if (a.flat_items)
-      return near ? launch_direct_as<CPT, uint32_t, true>(a, grid, st)
-                  : launch_direct_as<CPT, int64_t, true>(a, grid, st);
+      return near ? launch_direct_as<CPT, uint32_t, true>(a, grid, s, st)
+                  : launch_direct_as<CPT, int64_t, true>(a, grid, s, st);
   }
-  return near ? launch_direct_as<CPT, uint32_t, false>(a, grid, st)
-              : launch_direct_as<CPT, int64_t, false>(a, grid, st);
+  return near ? launch_direct_as<CPT, uint32_t, false>(a, grid, s, st)
+              : launch_direct_as<CPT, int64_t, false>(a, grid, s, st);
+}
+
+// Columns per thread: a warp's are consecutive, so that with more of them
+// fewer of the sectors that rows off the 32-byte grid split are shared between
+// warps, and they share each coset's twiddles; fewer leave fewer idle lanes at
+// the end of a row of B columns and need fewer registers.  The times below are
+// of x_1 passes of 24 x 24 matrices, relative to the Montgomery kernel before
+// unless two are compared.
+//
+// On the sector grid nothing is shared: one column over a flattened grid (no
+// idle lanes) up to 127 columns, two from 128 on: one / two / four columns, 8
+// words in: 72 columns .90 / 1.26 / 2.8, 104 .88 / .95 / 2.1, 128 .85 / .81 /
+// 1.8, 168 .86 / .87 / 1.6, 1024 .94 / .87 / .87, 8192 .98 / .93 / .94, 36864
+// .97 / .90 / .91; one word in (a broadcast), 16384 columns 4 : 2 .93.
+//
+// Off the grid a split sector costs a read as well where it leaves L2 before
+// its other part arrives, so it matters once the output is larger than L2
+// (kSplitBytes), and then
+//  - the columns of a row want to be few warps': four per thread from 384 on
+//    (545 columns, 8 words .96 / 1.05 / .95, 5 words 1.06 / 1.04 / .97), two
+//    from 129 on;
+//  - a row's warps want to be one CTA's: 97 to 127 columns two per thread on 64
+//    threads (97 columns, 4 words .75 of the flattened grid's time, 5 words
+//    .77), 49 to 63 one on 64 (4 words .82, 6 words .86), 73 to 95 one on 128,
+//    eight CTAs per SM (85 columns, 4 words .96 of 256 threads without that
+//    limit, 1.09 of 128 without it; 6 words .92 and .93);
+//  - the others, whose last warp would be nearly empty, stay flattened, with
+//    few CTAs at work, so that the other part of a sector is written soon: 65
+//    columns, per SM three CTAs of 128 threads with 8 words .78 of the time
+//    without a limit, 6 words .83; four with 5 words .88, five with 4 words
+//    .84, eight with 3 words .92.  With outputs that stay in L2 the limit
+//    costs (65 columns, 8 primes: 6 words .91, 4 words 1.05, 4 primes 1.22 and
+//    1.10).  Eight words take it up to 1023 columns (129 columns .86 against
+//    1.02 with two columns, 257 .92 and .99, 385 .91 and .98), six and seven up
+//    to 144 (129 columns, 7 words .87 and 1.00; 193 1.00 and .95).
+//
+// Blocks of columns (A > 1), interleaved output, and passes too small to fill
+// the chip take one column over a flattened grid.
+static DirectShape direct_shape(const TxArgs &a, int items, int nprimes) {
+  constexpr int64_t kSplitBytes = 128000000;
+  const bool flat_ok = a.A * a.B * items < ((int64_t)1 << 31) - kDirectThreads;
+  const DirectShape flat = {1, kDirectThreads, flat_ok, 0};
+  if (a.A != 1 || a.il_L || a.B < 8) return flat;
+  const int64_t row = a.out_row ? a.out_row : a.B;
+  const bool many = a.B * items * nprimes >= 152 * 4096;
+  const DirectShape one = {1, kDirectThreads, false, 0}, two = {2, kDirectThreads, false, 0},
+                    four = {4, kDirectThreads, false, 0};
+  if (row % 8 == 0) {
+    if (!many || a.B < 64 || (a.B < 128 && a.Lin > 1)) return flat;
+    return a.B < 128 ? one : a.Lin == 1 && a.B >= 8192 ? four : two;
+  }
+  if (4 * row * out_rows(a) * items * nprimes < kSplitBytes) {
+    if (!many || a.B < 64 || (a.B < 128 && a.Lin > 1)) return flat;
+    return a.B < 128 ? one : a.B >= 512 ? four : two;
+  }
+  const DirectShape capped = a.Lin <= 2   ? DirectShape{1, 128, true, 0}
+                             : a.Lin == 3 ? DirectShape{1, 256, true, 4}
+                                          : DirectShape{1, 128, true, a.Lin == 4 ? 5 : a.Lin == 5 ? 4 : 3};
+  if (flat_ok && a.B < (a.Lin == 8 ? 1024 : a.Lin >= 6 && a.B > 128 ? 145 : 0)) return capped;
+  if (a.B >= 384) return four;
+  if (a.B > 128) return two;
+  if (a.B > 96 && a.Lin < 7) return {2, 64, false, 0};
+  if (a.Lin <= 2 && flat_ok) return capped;
+  if (a.B >= 48 && a.B <= 64) return {1, 64, false, 0};
+  if ((a.B >= (a.Lin <= 5 ? 72 : 80) && a.B <= 96) || !flat_ok) return {1, 128, false, 8};
+  return capped;
 }
 
 static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
@@ -171,27 +268,10 @@ static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
   const bool window_ok = a.row_hi == 0 || (a.olp > 1 && a.olp == lp_in && a.row_lo % lp_in == 0);
   if (!a.inverse && a.Lin <= 8 && a.N <= kDirectTwSmem && rows_ok && window_ok &&
       (a.olp <= 1 || a.olp == lp_in)) {
-    // columns per thread: a warp's are consecutive, so that with more of them
-    // fewer of the sectors that rows off the 32-byte grid split are shared
-    // between warps, and they share each coset's twiddles; fewer leave fewer
-    // idle lanes at the end of a row of B columns and need fewer registers.
-    // x_1 passes in TB/s with 1 / 2 / 4 columns: 4 words, rows of 1369 columns
-    // 5.1 / 5.5 / 5.6, 3 words, 943 columns 5.4 / 5.1 / 5.7, 2 words, 441
-    // columns 4.6 / 5.9 / 5.4, 7 words, 193 columns 3.6 / 5.2 / 4.3, 5 words,
-    // 97 columns 4.2 / 4.7 / 2.3, 4 words, 73 columns 4.8 / 4.2 / 3.0; on the
-    // grid (1024 columns) 5.0 / 6.0 / 5.9.  One column, over a flattened grid,
-    // where the columns are not one block (A > 1, interleaved output) or the
-    // pass is too small to fill the chip otherwise.
-    int cpt = 1;
-    bool flat = ncols * items < ((int64_t)1 << 31) - kDirectThreads;
-    if (a.A == 1 && !a.il_L && a.B >= 64 && a.B * items * nprimes >= 152 * 4096) {
-      const bool split = (a.out_row ? a.out_row : a.B) % 8;  // rows off the 32-byte grid
-      flat = false;
-      cpt = lp_in <= 4 && a.B >= (split ? 512 : 8192) ? 4 : lp_in > 4 || a.B >= 128 ? 2 : 1;
-    }
+    const DirectShape shape = direct_shape(a, items, nprimes);
     // short rows: one grid axis over (item, column) pairs, so that rows
     // shorter than a CTA, or a row's last CTA, leave no threads idle
-    a.flat_items = flat ? items : 0;
+    a.flat_items = shape.flat ? items : 0;
     // few columns in all (a job's first pass): cut each column's cosets into
     // groups until the grid holds about 152 x 1024 threads
     a.flat_groups = 1;
@@ -205,10 +285,10 @@ static int launch_pass(TxArgs a, int items, int nprimes, cudaStream_t st) {
       while (g > 1 && ncols * items * g >= ((int64_t)1 << 31) - 256) --g;
       a.flat_groups = (int)std::max<int64_t>(1, g);
     }
-    switch (cpt) {
-      case 4: return launch_direct<4>(a, ncols, items, nprimes, st);
-      case 2: return launch_direct<2>(a, ncols, items, nprimes, st);
-      default: return launch_direct<1>(a, ncols, items, nprimes, st);
+    switch (shape.cpt) {
+      case 4: return launch_direct<4>(a, ncols, items, nprimes, shape, st);
+      case 2: return launch_direct<2>(a, ncols, items, nprimes, shape, st);
+      default: return launch_direct<1>(a, ncols, items, nprimes, shape, st);
     }
   }
   // Ct: columns per CTA, a power of two with N * (Ct + 1) words <= 64 KB.

@@ -82,11 +82,12 @@ PD_HD int out_rows(const TxArgs &a) { return a.row_hi ? a.row_hi - a.row_lo : a.
 //  - stores go to a base pointer that is the same for the whole CTA plus a
 //    running offset per output row, 32-bit wherever the output of a CTA's
 //    prime (flat grid) or item fits in 4 GB (Off = uint32_t, launch_pass);
-//  - the cosets whose rows are all stored take no per-store predicate.
+//  - the cosets whose rows are all stored take no predicate but that of a
+//    thread's second to fourth column.
 // Plans keep D_v <= n d_v, so with at most 8 inputs (d_v <= 7) and n <= 32 a
 // circle has N <= 256 points; launch_pass sends anything longer to the
 // shared-memory pass kernel.
-constexpr int kDirectThreads = 256;
+constexpr int kDirectThreads = 256;  // at most
 constexpr int kDirectTwSmem = 256;
 
 // x w mod p in [0, p), tw = (w, floor(w 2^32 / p)), any x < 2^32.
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
   const uint2 *tw = a.tws + (size_t)q * a.tw_len + a.tw_off;
   // every twiddle index used is below N (j < N / LP and e < LP), and
   // N <= kDirectTwSmem (launch_pass); staged before any thread leaves
-  for (int i = threadIdx.x; i < a.N; i += kDirectThreads) s_tw[i] = __ldg(tw + i);
+  for (int i = threadIdx.x; i < a.N; i += blockDim.x) s_tw[i] = __ldg(tw + i);
   __syncthreads();
   const uint32_t p = a.mod[q].p;
   const int64_t ncols = a.A * a.B;
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(kDirectThreads) coltx_direct_kernel(TxArgs a) 
   int grp = 0;
   int64_t item = blockIdx.y;
   // the first column, the others 32 apart
-  int64_t first = (int64_t)blockIdx.x * kDirectThreads * CPT + warp * (32 * CPT) + lane;
+  int64_t first = (int64_t)blockIdx.x * blockDim.x * CPT + warp * (32 * CPT) + lane;
   // the CTA's output: its prime's, or its item's
   char *base = reinterpret_cast<char *>(a.out + (int64_t)blockIdx.z * a.out_prime_stride);
   if (FLAT) {  // items * ncols * groups < 2^31 (launch_pass)
