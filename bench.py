@@ -681,8 +681,8 @@ def structured_leg(st, hbm_peak, derived_upd):
 def run_ours(args, world, rank, local):
     import torch
     from paper_2010_12117_gb300 import synth
-    from paper_2010_12117_gb300.binding import condense_columns, probe_int_peaks
-    from paper_2010_12117_gb300.runner import BatchedRunner, PlainRunner, StageTimer
+    from paper_2010_12117_gb300.binding import condense_columns, condense_launch, probe_int_peaks
+    from paper_2010_12117_gb300.runner import BatchedRunner, PlainRunner, StageTimer, condense_updates
 
     torch.cuda.set_device(local)
     dev_props = torch.cuda.get_device_properties(local)
@@ -773,6 +773,13 @@ def run_ours(args, world, rank, local):
     bytes_by_order = {}
     for pm, pl in zip(plain.mats, plain.plans):
         bytes_by_order[pm.n] = bytes_by_order.get(pm.n, 0.0) + float(pl.P * pl.G) * (4 * pm.n * pm.n + 4)
+    # updates of each order's launches by the columns their kernels take at a time
+    upd_by_columns = {}
+    for pm, pl, chunks in zip(plain.mats, plain.plans, plain.chunks):
+        by = upd_by_columns.setdefault(pm.n, {})
+        for lo, hi in chunks:
+            cols = condense_launch(pm.n, (hi - lo) * pl.G, max(pl.primes[lo:hi]))[1]
+            by[cols] = by.get(cols, 0.0) + float((hi - lo) * pl.G * condense_updates(pm.n))
     plain.close()
     del plain
 
@@ -785,8 +792,8 @@ def run_ours(args, world, rank, local):
     sms = dev_props.multi_processor_count
     sm_mhz = clocks.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     lanes = sms * 64 * sm_mhz * 1e6  # IMAD lanes per second (64 per SM per clock)
-    # The condensation kernel of order n takes its elimination steps two,
-    # three or four at a time (condense_columns).  One element update of a step pair
+    # The condensation kernel of a launch takes its elimination steps two,
+    # three or four at a time (condense_launch).  One element update of a step pair
     # (two algorithmic updates) issues three 32x32->64-bit multiply-adds and
     # the REDC's IMAD and IMAD.HI; the pipe costs ncu measures on the probes
     # (a wide multiply-add or an IMAD.HI holds the FMA-heavy pipe two slots,
@@ -797,14 +804,12 @@ def run_ours(args, world, rank, local):
     # third's rate is the triple's scaled by the slots.
     slots = {2: 4.5, 3: 11.0 / 3.0, 4: 13.0 / 4.0}
     probe_upd = {2: 2.0 * pair_s, 3: 3.0 * triple_s, 4: 4.0 * triple_s * 11.0 / 13.0}
-    step_of = {n_: condense_columns(n_) for n_ in range(1, 33)}
-
-    def model_peak(n_):
-        return lanes / slots[step_of[n_]]
+    def model_peak(n_):  # large launches
+        return lanes / slots[condense_columns(n_)]
     single_step_upd = lanes / 6.0  # the single-step kernel's model (6 slots), kept for comparison
     peak_src = (f"derived: {sms} SMs x 64 IMAD/clk x {sm_mhz:.0f} MHz / IMAD slots per update "
-                "of each order's pass (4.5 for a step pair, 11/3 for a step triple, 13/4 for two nested pairs), weighted by "
-                "each order's updates")
+                "of each launch's pass (4.5 for a step pair, 11/3 for a step triple, 13/4 for two nested pairs), weighted "
+                "by its updates")
     # per order: the update rate against its integer-pipe peak, the byte rate
     # against HBM, and the time either bound alone allows; the sum of those
     # times over the sum of the measured ones is the kernel's fraction of its
@@ -814,16 +819,18 @@ def run_ours(args, world, rank, local):
     t_model = t_probe = upd_all = 0.0
     for n_, (ms_, upd) in sorted(ptimer.tag_ms("condense").items()):
         byt = bytes_by_order[n_]
-        pk = model_peak(n_)
+        by = upd_by_columns[n_]
+        pk = upd / sum(u * slots[c] / lanes for c, u in by.items())
+        probe_pk = upd / sum(u / probe_upd[c] for c, u in by.items())
         tb = max(upd / pk, byt / (hbm_peak * 1e9))
         t_bound += tb
         t_meas += ms_ * 1e-3
         t_model += upd / pk
-        t_probe += upd / probe_upd[step_of[n_]]
+        t_probe += upd / probe_pk
         upd_all += upd
-        by_order[str(n_)] = {"ms": ms_, "steps_per_pass": step_of[n_], "Gupdate_s": upd / (ms_ * 1e-3) / 1e9,
+        by_order[str(n_)] = {"ms": ms_, "steps_per_pass": max(by, key=by.get), "Gupdate_s": upd / (ms_ * 1e-3) / 1e9,
                              "alu_frac": upd / (ms_ * 1e-3) / pk,
-                             "alu_frac_of_probe": upd / (ms_ * 1e-3) / probe_upd[step_of[n_]],
+                             "alu_frac_of_probe": upd / (ms_ * 1e-3) / probe_pk,
                              "alu_frac_of_single_step_peak": upd / (ms_ * 1e-3) / single_step_upd,
                              "hbm_frac": byt / (ms_ * 1e-3) / (hbm_peak * 1e9),
                              "bound": "alu" if upd / pk >= byt / (hbm_peak * 1e9) else "hbm"}
