@@ -421,7 +421,9 @@ int polydet_batch_test_drop_copies(polydet_batch_t batch, int on);
  * only: no device call. */
 int polydet_team_size(int n);
 /* Columns of the pivot blocks the condensation kernels of order n eliminate
- * by (2 or 3); POLYDET_EINVAL outside 1..32.  Host only. */
+ * by (2 or 3; two nested 2 x 2 blocks count as 2); POLYDET_EINVAL outside
+ * 1..32.  Kept for its callers: polydet_condense_columns and
+ * polydet_condense_launch give the columns eliminated at a time.  Host only. */
 int polydet_condense_steps(int n);
 /* Columns the condensation kernel of large launches of order n eliminates at a
  * time: 2 or 3, or 4 where two 2 x 2 pivot blocks are applied together (the

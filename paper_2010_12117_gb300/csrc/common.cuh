@@ -46,7 +46,7 @@ struct polydet_plan_s {
   int full;                        // 1: full power-of-two grid + inverse NTT
   int itab_off[POLYDET_MAX_VARS];  // node grid: offset of variable v's interpolation tables
   int itab_len;                    // node grid: their words per prime
-  uint32_t *d_itab;                // [P][itab_len] (layout in plan.cu, Montgomery forms)
+  uint32_t *d_itab;                // [P][itab_len] (layout: CiTab; Montgomery forms)
   int tw_len;                      // sum_v N_v: twiddles per prime
   uint32_t primes[POLYDET_MAX_PRIMES];
   uint32_t roots[POLYDET_MAX_PRIMES][POLYDET_MAX_VARS];

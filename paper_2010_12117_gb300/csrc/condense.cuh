@@ -2,8 +2,8 @@
 //
 // A team of T consecutive lanes owns one matrix: lane t holds the columns
 // j = t - s, t - s + T, t - s + 2T, ... in registers (one lane for n <= 13, two,
-// four or eight above; the per-order T and the CTAs per SM the
-// kernel is compiled for are the table of teams.cuh).  The s = T ceil(n/T) - n
+// four or eight above and in some small launches; T and the CTAs per SM the
+// kernel is compiled for are the tables of teams.cuh).  The s = T ceil(n/T) - n
 // padding slots (j < 0) sit in the first block of T columns, which drops out
 // of the elimination after its first steps; in the last block they would be
 // computed and discarded at almost every step.  Every index into the register

@@ -134,7 +134,7 @@ static size_t direct_reserve_bytes(int ctas) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   // static twiddles and the 1 KB the system keeps per CTA count as well
-  return (size_t)per_sm / (ctas + 1) + 256 - kDirectTwSmem * sizeof(uint2) - 1024;
+  return (size_t)std::max(0, per_sm / (ctas + 1) + 256 - (int)(kDirectTwSmem * sizeof(uint2)) - 1024);
 }
 
 template <int CPT, class Off, bool FLAT>

@@ -20,8 +20,8 @@
 //   18 287 -> 244   19 327 -> 297   20 390 -> 338   21 450 -> 414   22 507 -> 474
 //   23 573 -> 531   24 643 -> 570   25 991 -> 667   26 1062 -> 804  27 1171 -> 858
 //   28 1223 -> 962  29 1407 -> 1312 30 1524 -> 1417 31 1684 -> 1436 32 1777 -> 1592
-// Quads (five products and one reduction for four columns) win from order 14
-// on, where the trailing matrix is large enough to pay for their panel.  Four
+// Quads (five products and one reduction for four columns) win at order 10 and
+// from 14 on, where the trailing matrix is large enough to pay for their panel.  Four
 // lanes beat eight up to order 28: the panel is computed once per lane, and
 // the registers that spill (up to 700 bytes at order 28) cost less; from 29
 // on they cost more (order 29: 1454 with four lanes).  Folding the pivots at
