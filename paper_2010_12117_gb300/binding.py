@@ -253,6 +253,14 @@ _shape_consts: dict = {}
 _shape_lock = threading.Lock()
 
 
+def plan_cache_clear() -> None:
+    """Give back what is kept per shape: the library's idle device tables and the constants kept here (live plans
+    keep theirs)."""
+    _check(lib().polydet_plan_cache_clear(), "polydet_plan_cache_clear")
+    with _shape_lock:
+        _shape_consts.clear()
+
+
 class Plan:
     """A polydet plan: n x n matrices in len(degs) variables, entry degree
     <= degs[v] in x_v, over the first ``nprimes`` primes of the table; node
@@ -291,7 +299,7 @@ class Plan:
         self.items = self.entries - 1 if info.unique >= 0 else self.entries  # evaluated entries
         # primes, roots and node exponents depend on the shape alone: asked for
         # once per shape (three library calls and hundreds of list items), kept
-        # for the most recent ones
+        # for the most recent ones until plan_cache_clear()
         key = (self.n, self.d, self.D, self.P, self.full_grid)
         consts = _shape_consts.get(key)
         if consts is None:
@@ -609,7 +617,8 @@ def probe_int_peaks(stream=None) -> tuple[float, float, float, float]:
 
 
 def condense_steps(n: int) -> int:
-    """Columns of the pivot blocks of the condensation kernels of order n (2 or 3)."""
+    """Columns of the pivot blocks of the condensation kernels of order n (2 or 3; two 2 x 2 blocks count as 2).
+    condense_columns and condense_launch say what a kernel eliminates at a time; this stays for its callers."""
     t = lib().polydet_condense_steps(int(n))
     if t < 1:
         _check(t, "polydet_condense_steps")
