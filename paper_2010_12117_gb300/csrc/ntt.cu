@@ -203,7 +203,10 @@ static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes,
 // idle lanes) up to 127 columns, two from 128 on: one / two / four columns, 8
 // words in: 72 columns .90 / 1.26 / 2.8, 104 .88 / .95 / 2.1, 128 .85 / .81 /
 // 1.8, 168 .86 / .87 / 1.6, 1024 .94 / .87 / .87, 8192 .98 / .93 / .94, 36864
-// .97 / .90 / .91; one word in (a broadcast), 16384 columns 4 : 2 .93.
+// .97 / .90 / .91.  Long rows of at most four words take four, which the whole
+// circle hardly tells from two (4 words, 36864 columns .96 and .97) but one
+// word and slabs do: one word, 16384 columns 257 us against 278; a 15 x 15
+// matrix of 1.1e8 nodes streamed in slabs, 4 words, 86.0 ms in all against 87.5.
 //
 // Off the grid a split sector costs a read as well where it leaves L2 before
 // its other part arrives, so it matters once the output is larger than L2
@@ -239,7 +242,7 @@ static DirectShape direct_shape(const TxArgs &a, int items, int nprimes) {
                     four = {4, kDirectThreads, false, 0};
   if (row % 8 == 0) {
     if (!many || a.B < 64 || (a.B < 128 && a.Lin > 1)) return flat;
-    return a.B < 128 ? one : a.Lin == 1 && a.B >= 8192 ? four : two;
+    return a.B < 128 ? one : a.Lin <= 4 && a.B >= 8192 ? four : two;
   }
   if (4 * row * out_rows(a) * items * nprimes < kSplitBytes) {
     if (!many || a.B < 64 || (a.B < 128 && a.Lin > 1)) return flat;

@@ -73,9 +73,10 @@ def test_outputs_larger_than_l2(lin, rows):
     _check(lin, rows, large=True)
 
 
-def test_broadcast_of_one_word():
-    """One coefficient of x_1, rows on the grid and long: four columns per thread."""
-    _check(1, 8192)
+@pytest.mark.parametrize("lin", [1, 4])
+def test_long_rows_on_the_grid(lin):
+    """At most four coefficients of x_1: four columns per thread."""
+    _check(lin, 8192)
 
 
 @pytest.mark.parametrize("lin", [2, 3, 5, 8])
@@ -84,13 +85,13 @@ def test_power_of_two_grid(lin, rows):
     _check(lin, rows, full=True)
 
 
-@pytest.mark.parametrize("rows", [609, 1025])
-def test_windows_of_rows(rows):
-    """Slabs of nodes of x_1 (rows off the grid; rows padded to it) against one evaluation of all of them."""
+@pytest.mark.parametrize("tail", [(608,), (1024,), (96, 84)])
+def test_windows_of_rows(tail):
+    """Slabs of nodes of x_1 (rows of 609 nodes; of 1025 and 8245, padded to the grid) against one evaluation of all
+    of them."""
     from paper_2010_12117_gb300.binding import Plan
-    lin, d2 = 4, -(-(rows - 1) // N)
-    pl = Plan(N, (lin - 1, d2), 1, det_degs=(26, rows - 1))
-    rng = np.random.default_rng(rows)
+    pl = Plan(N, (3,) + tuple(-(-x // N) for x in tail), 1, det_degs=(26,) + tail)
+    rng = np.random.default_rng(sum(tail))
     c = torch.from_numpy(rng.integers(-2 ** 31, 2 ** 31, N * N * pl.E).astype(np.int32)).cuda()
     evals = torch.empty(N * N * pl.G, dtype=torch.int32, device="cuda")
     want, got = (torch.empty(pl.G, dtype=torch.int32, device="cuda") for _ in range(2))
