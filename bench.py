@@ -37,10 +37,10 @@ METRIC = ("exact poly determinants/sec and mod-p n×n dets/sec; IMAD % and HBM G
 # capture), valid only for the code it was taken on: digests of the
 # kernel's sources with comments and blank space removed; the bench reports
 # traffic null once they change.
-CONDENSE_TRAFFIC = {"ratio": 1.0133, "fmaheavy_active": 0.716,
-                    "sources": {"paper_2010_12117_gb300/csrc/condense.cuh": "b0dcc202ebcb755b",
-                                "paper_2010_12117_gb300/csrc/modarith.cuh": "b36f048e62c9ded4",
-                                "paper_2010_12117_gb300/csrc/teams.cuh": "2b54f7c70ebf5672"}}
+CONDENSE_TRAFFIC = {"ratio": 1.0147, "fmaheavy_active": 0.681,
+                    "sources": {"paper_2010_12117_gb300/csrc/condense.cuh": "d37077192686c68d",
+                                "paper_2010_12117_gb300/csrc/modarith.cuh": "d76fd317751b6f64",
+                                "paper_2010_12117_gb300/csrc/teams.cuh": "900b45829c0d6ba9"}}
 
 
 def _code_digest(path: str) -> str:
@@ -66,12 +66,12 @@ def _traffic_ratio():
 # coefficients, from one ncu capture, valid for the sources it was taken on.
 CRT_PIPE = {"fmaheavy_active": {11: 0.843},
             "sources": {"paper_2010_12117_gb300/csrc/crt.cu": "b7f51ef1688995fc",
-                        "paper_2010_12117_gb300/csrc/modarith.cuh": "b36f048e62c9ded4"}}
-# The same for the x_1 pass (coltx_direct_kernel<4, 2>) of the node-grid
+                        "paper_2010_12117_gb300/csrc/modarith.cuh": "d76fd317751b6f64"}}
+# The same for the x_1 pass (coltx_direct_kernel<4, 4>) of the node-grid
 # evaluation (37^3 nodes, 20 primes), the pass that moves its bytes.
-EVAL_PIPE = {"fmaheavy_active": 0.779,
-             "sources": {"paper_2010_12117_gb300/csrc/ntt_direct.cuh": "cca188a993a99705",
-                         "paper_2010_12117_gb300/csrc/modarith.cuh": "b36f048e62c9ded4"}}
+EVAL_PIPE = {"fmaheavy_active": 0.577,
+             "sources": {"paper_2010_12117_gb300/csrc/ntt_direct.cuh": "51996db02328e368",
+                         "paper_2010_12117_gb300/csrc/modarith.cuh": "d76fd317751b6f64"}}
 
 
 WORKLOAD = ("batched: 256 matrices, n~U[4,24], k~U{1,2,3}, d_v~U[1,4], density~U[0.3,1.0], "

@@ -223,9 +223,9 @@ static int launch_direct(const TxArgs &a, int64_t ncols, int items, int nprimes,
 //    few CTAs at work, so that the other part of a sector is written soon: 65
 //    columns, per SM three CTAs of 128 threads with 8 words .78 of the time
 //    without a limit, 6 words .83; four with 5 words .88, five with 4 words
-//    .84, eight with 3 words .92.  With outputs that stay in L2 the limit
-//    costs (65 columns, 8 primes: 6 words .91, 4 words 1.05, 4 primes 1.22 and
-//    1.10).  Eight words take it up to 1023 columns (129 columns .86 against
+//    .84, four of 256 with 3 words .88.  With outputs that stay in L2 the
+//    limit costs (65 columns, 8 primes: 6 words .91, 4 words 1.05, 4 primes 1.22
+//    and 1.10).  Eight words take it up to 1023 columns (129 columns .86 against
 //    1.02 with two columns, 257 .92 and .99, 385 .91 and .98), six and seven up
 //    to 144 (129 columns, 7 words .87 and 1.00; 193 1.00 and .95).
 //
